@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(NT, batch_min_blocks(NT))
       stage_plain<TR, TW, NT, true>(v, gm, S);
     // the threshold rows and round keys stay from the block's previous item
     // when it had the same replica (and gate)
-    if (rep != s_tab_rep || g != s_tab_g) fill_rows2(Tb, R.table24, g);
+    if (rep != s_tab_rep || g != s_tab_g) fill_rows2(Tb, R.table24, g, NT);
     if (rep != s_key_rep && threadIdx.x < 10) {
       s_keys.k[threadIdx.x] = R.keys.k[threadIdx.x];
     }
@@ -289,9 +289,9 @@ __global__ void __launch_bounds__(NT, batch_min_blocks(NT))
     if constexpr (kWalkShape) {
       if (walk) {
         if (rec)
-          colour0_walk<RNG_WORDS, CMP64, TR, TW, NT, true, 1>(v, gm, S, Tb, cnt, s_hist4);
+          colour0_walk<RNG_WORDS, CMP64, TR, TW, NT, true, 2>(v, gm, S, Tb, cnt, s_hist4);
         else
-          colour0_walk<RNG_WORDS, CMP64, TR, TW, NT, false, 1>(v, gm, S, Tb, cnt, nullptr);
+          colour0_walk<RNG_WORDS, CMP64, TR, TW, NT, false, 2>(v, gm, S, Tb, cnt, nullptr);
       }
     }
     if (!walk)
@@ -333,9 +333,9 @@ __global__ void __launch_bounds__(NT, batch_min_blocks(NT))
     if constexpr (kWalkShape) {
       if (walk) {
         if (rec)
-          colour1_walk<RNG_WORDS, CMP64, TR, TW, NT, true, 1>(v, gm, S, Tb, cnt, s_hist4);
+          colour1_walk<RNG_WORDS, CMP64, TR, TW, NT, true, 2>(v, gm, S, Tb, cnt, s_hist4);
         else
-          colour1_walk<RNG_WORDS, CMP64, TR, TW, NT, false, 1>(v, gm, S, Tb, cnt, nullptr);
+          colour1_walk<RNG_WORDS, CMP64, TR, TW, NT, false, 2>(v, gm, S, Tb, cnt, nullptr);
       }
     }
     if (!walk)

@@ -161,9 +161,9 @@ __device__ __forceinline__ void split_draws(const Words4& u, const Words4& p, ui
   if (RNG_WORDS == 1) {
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
-      const uint64_t prod = (uint64_t)uw[a] * (uint64_t)(q - 1u);
-      kk[a] = (uint32_t)(prod >> 32);
-      acc[a] = (uint32_t)prod;
+      asm("{\n\t.reg .b64 t;\n\tmul.wide.u32 t, %2, %3;\n\tmov.b64 {%0, %1}, t;\n\t}"
+          : "=r"(acc[a]), "=r"(kk[a])
+          : "r"(uw[a]), "r"(q - 1u));
     }
   } else {
     const uint32_t pw[4] = {p.x, p.y, p.z, p.w};

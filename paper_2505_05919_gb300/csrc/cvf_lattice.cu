@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kThreads, kSweepBlocksPerSM)
       finalize_step<true>(*A.vol, ctl, A.ring, A.ring_cap, A.keys);
     return;
   }
-  fill_rows2(Tb, A.table24, g);
+  fill_rows2(Tb, A.table24, g, kThreads);
   fill_prop2(Tb, A.q);
   const long long N = (long long)A.L * A.L;
   StepView<KeysRound> v;
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(kThreads) k_layer(LatticeArgs A, int launch) {
   const long long step = ctl->sweep;
   const int g = ctl->next_g;
   const bool rec = s_rec != 0;
-  fill_rows2(Tb, A.table24, g);
+  fill_rows2(Tb, A.table24, g, kThreads);
   fill_prop2(Tb, A.q);
   if (threadIdx.x < 8) s_hist[threadIdx.x] = 0;
   __syncthreads();
@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(kThreads) k_layer(LatticeArgs A, int launch) {
     uint32_t pk = 0;
 #pragma unroll
     for (int hi = 0; hi < 2; ++hi) {
-      uint32_t w = hi ? (own >> 16) : (own & 0xFFFFu);
+      uint32_t w = twice(own, hi != 0);
       const uint32_t c = y * L + 2u * p + (uint32_t)hi;
       uint32_t acc[4], kk[4];
       cell_draws<RNG_WORDS>(c, s_lo, s_hi, A.keys, A.q, acc, kk);
@@ -557,9 +557,18 @@ __global__ void __launch_bounds__(kThreads) k_layer(LatticeArgs A, int launch) {
         // the draws of arm a, selected without indexing the arrays at run time
         const uint32_t ua = (a == 0) ? acc[0] : (a == 1) ? acc[1] : (a == 2) ? acc[2] : acc[3];
         const uint32_t ka = (a == 0) ? kk[0] : (a == 1) ? kk[1] : (a == 2) ? kk[2] : kk[3];
-        w = update_arm2<CMP64>(w, partner_operand(pa), ua, ka, (uint32_t)a, Tb, pk);
+        const uint32_t p2 = (pa >> 16) * (0x10001u << (4 * a));
+        // block-uniform: the arm a constant in each call
+        if (a == 0)
+          w = update_arm2<CMP64, 0>(w, p2, ua, ka, A.q, Tb, pk);
+        else if (a == 1)
+          w = update_arm2<CMP64, 1>(w, p2, ua, ka, A.q, Tb, pk);
+        else if (a == 2)
+          w = update_arm2<CMP64, 2>(w, p2, ua, ka, A.q, Tb, pk);
+        else
+          w = update_arm2<CMP64, 3>(w, p2, ua, ka, A.q, Tb, pk);
       }
-      out = hi ? ((out & 0xFFFFu) | (w << 16)) : ((out & 0xFFFF0000u) | w);
+      out = __byte_perm(out, w, hi ? 0x5410u : 0x3254u);
     }
     cnt.add(pk);
     dst[wi] = out;

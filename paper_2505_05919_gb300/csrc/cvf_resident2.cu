@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(kResBlock) k_resident2(LatticeArgs A, long lon
     const bool rec = step_recorded(every, step);
     const int g = *next_g0;
     if (g != g_cur) {  // uniform over the CTA's sweepers
-      fill_rows2(Tb, A.table24, g);
+      fill_rows2(Tb, A.table24, g, kResThreads);
       g_cur = g;
     }
     if (rank == 0 && threadIdx.x < 3) s_acc[threadIdx.x] = 0;

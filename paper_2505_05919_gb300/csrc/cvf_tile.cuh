@@ -19,103 +19,112 @@ namespace cvf {
 
 // Shared tables of one (lattice, step): the proposal for the current q and
 // the threshold rows of the current gate.
-//   prop[8 k + sigma] = {sigma * 0x11111111, ((sigma + 1 + k) mod q) *
-//                       0x11111111} for k < 7 (sigma and sigma' in every
-//                       nibble; k <= q - 2 <= 6): both words an update needs
-//                       in one 8-byte load at byte offset 64 k + 8 sigma
-//   rows[9 ps + pp]   = {T - 1, packed count change} for the nibble counts ps,
-//                       pp of update_arm2 (entries no move can reach are 0);
-//                       an accepted move adds the change (1 << 20) +
-//                       ((dN_HB + 1) << 10) + dN_sigma + 3
-//   T64[9 ps + pp]    = T (the 64-bit compare, when some T is 0)
-constexpr int kRows2 = 72;
+//   prop[q k + sigma] = sigma in the low four nibbles, 7 ^ sigma' (sigma' =
+//                       (sigma + 1 + k) mod q) in the high four (k <= q - 2
+//                       <= 6); for q = 6 the 30 entries lie in 30 different
+//                       banks
+//   next[q k + sigma] = sigma' in every nibble
+//   rows              = the pairs {T - 1, packed count change} for the sums of
+//                       update_arm2, one table for an arm in an even nibble
+//                       and one for an odd one; an accepted move adds the
+//                       change (1 << 20) + ((dN_HB + 1) << 10) + dN_sigma + 3.
+//                       {0, 0} where no move can reach the pair, or where T =
+//                       0 (no draw is below it): the kernels of a table that
+//                       holds a T = 0 also ask for a nonzero change (CMP64).
+//                       Two copies, the second an odd number of words after
+//                       the first: the thresholds of the even lanes lie in the
+//                       even banks, those of the odd lanes in the odd ones.
+constexpr int kRowWords = 2 * (2 * (1 + 4 + 16 + 64) + 1);  // pairs up to the largest sums
+constexpr int kRowCopy = 2 * kRowWords + 1;                 // words from one copy to the next
 struct Tables2 {
-  uint2 rows[kRows2];
-  uint2 prop[64];
-  unsigned long long T64[kRows2];
+  uint32_t rows[2 * kRowCopy];
+  uint32_t prop[64];
+  uint32_t next[64];
 };
 
 // Proposal part of the tables (depends on q only).
 __device__ __forceinline__ void fill_prop2(Tables2& Tb, uint32_t q) {
   for (int e = threadIdx.x; e < 64; e += blockDim.x) {
-    const uint32_t k = (uint32_t)e >> 3, s = (uint32_t)e & 7u;
-    uint32_t v = 0u;
-    if (s < q && k + 1u < q) {
-      uint32_t sp = s + 1u + k;
-      while (sp >= q) sp -= q;
-      v = sp * 0x11111111u;
-    }
-    Tb.prop[e] = make_uint2(s * 0x11111111u, v);
+    const uint32_t k = (uint32_t)e / q, s = (uint32_t)e - k * q;
+    uint32_t sp = s + 1u + k;  // entries with k > q - 2 are never read
+    while (sp >= q) sp -= q;
+    Tb.prop[e] = s * 0x1111u + (sp ^ 7u) * 0x11110000u;
+    Tb.next[e] = sp * 0x11111111u;
   }
 }
 
 // Threshold part from a [g][(dN_HB+1)*8 + dN_sigma+3] table of 24 per gate.
-// Entry 9 ps + pp: ps = A_s + 4 b_s with A_s <= 3 the arms differing from
-// sigma and b_s = [partner != sigma]; pp = A_p + 4 b_p with 1 <= A_p <= 4
-// for sigma' -- so b_s = ps >> 2, A_s = ps & 3, b_p = [pp >= 5], A_p = pp -
-// 4 b_p, dN_HB = b_s - b_p and dN_sigma = A_s - A_p + 1.
-__device__ __forceinline__ void fill_rows2(Tables2& Tb, const unsigned long long* table24, int g) {
-  for (int i = threadIdx.x; i < kRows2; i += blockDim.x) {
-    const int ps = i / 9, pp = i % 9;
-    const int bs = ps >> 2, as = ps & 3, bp = (pp >= 5) ? 1 : 0, ap = pp - 4 * bp;
-    if (ap < 1) {  // unreachable: arm a itself always differs from sigma'
-      Tb.rows[i] = make_uint2(0u, 0u);
-      Tb.T64[i] = 0ull;
-      continue;
+// Pair i holds four sums of two bits each; the partner's is the first for an
+// arm in an even nibble and the third for one in an odd nibble (update_arm2):
+// it is dN_HB + 1, and the other three add up to dN_sigma + 3.  Called by the
+// block's first `threads` threads.
+__device__ __forceinline__ void fill_rows2(Tables2& Tb, const unsigned long long* table24, int g,
+                                           int threads) {
+  for (int i = threadIdx.x; i < kRowWords; i += threads) {
+    const int odd = i >= kRowWords / 2 ? 1 : 0, n = i - odd * (kRowWords / 2);
+    const int f0 = n & 3, f1 = (n >> 2) & 3, f2 = (n >> 4) & 3, f3 = (n >> 6) & 3;
+    const int hb = odd ? f2 : f0, dc = f1 + f3 + (odd ? f0 : f2);
+    uint32_t thr = 0u, change = 0u;
+    if (f0 < 3 && f1 < 3 && f2 < 3 && f3 < 3) {  // each sum is 0, 1 or 2
+      const unsigned long long t = table24[g * 24 + hb * 8 + dc];
+      if (t) {
+        thr = (uint32_t)(t - 1ull);
+        change = (1u << 20) + ((uint32_t)hb << 10) + (uint32_t)dc;
+      }
     }
-    const int dhb = bs - bp, dc = as - ap + 1;
-    const unsigned long long t = table24[g * 24 + (dhb + 1) * 8 + (dc + 3)];
-    Tb.rows[i] = make_uint2((uint32_t)(t - 1ull),  // every t >= 1 unless 64-bit compares
-                            (1u << 20) + ((uint32_t)(dhb + 1) << 10) + (uint32_t)(dc + 3));
-    Tb.T64[i] = t;
+    uint32_t* pair = Tb.rows + 2 * i;
+    pair[0] = pair[kRowCopy] = thr;
+    pair[1] = pair[kRowCopy + 1] = change;
   }
 }
 
-constexpr uint32_t kNib1 = 0x11111111u;   // 1 in every nibble
-constexpr uint32_t kGuard = 0x88888888u;  // bit 3 of every nibble
-
-// The partner operand of update_arm2 from a partner value pa placed at bits
-// 16..18: pa copied into nibbles 4..7 and bit 3 of every nibble set.
-__device__ __forceinline__ uint32_t partner_operand(uint32_t pa16) {
-  return pa16 * 0x1111u + kGuard;
+// A cell's word (low or high half of a lattice word) in both halves.
+__device__ __forceinline__ uint32_t twice(uint32_t word, bool hi) {
+  return __byte_perm(word, 0u, hi ? 0x3232u : 0x1010u);
 }
 
-// Metropolis update of arm a of a cell word w (sigma_b in nibble b, b =
-// 0..3, nibbles 4..7 zero) with draw u and proposal offset k (Sec. II.C,
-// Eq. H).  x is the partner operand: the partner value (arm a^1 of the
-// neighbour in direction a) in nibbles 4..7 and bit 3 of every nibble set.
-// For v = sigma or sigma' (v R = v in every nibble), t = w ^ v R ^ x holds
-// in each nibble 8 + (nibble ^ v), so f(v) = (t - R) & M has bit 3 of nibble
-// b set iff nibble b differs from v (no borrow crosses a nibble).  popc f
-// (sigma) = A_s + 4 b_s and popc f(sigma') = A_p + 4 b_p index the rows
-// directly.  ARM >= 0 fixes a at compile time; ARM = -1 takes it from a_rt.
-template <bool CMP64, int ARM = -1>
-__device__ __forceinline__ uint32_t update_arm2(uint32_t w, uint32_t x, uint32_t u, uint32_t k,
-                                                uint32_t a_rt, const Tables2& Tb, uint32_t& pk) {
-  const uint32_t a = (ARM >= 0) ? (uint32_t)ARM : a_rt;
-  // 8 sigma: the byte offset of sigma's entry in a proposal table row
-  uint32_t s8;
-  if constexpr (ARM == 0)
-    s8 = (w << 3) & 0x38u;
-  else if constexpr (ARM > 0)
-    s8 = (w >> (4 * ARM - 3)) & 0x38u;
-  else
-    s8 = ((w >> (4u * a)) & 7u) << 3;
-  const uint2 pr = *reinterpret_cast<const uint2*>(reinterpret_cast<const char*>(Tb.prop) +
-                                                   (k << 6) + s8);
-  const uint32_t sR = pr.x;   // sigma in every nibble
-  const uint32_t spR = pr.y;  // sigma' in every nibble
-  const uint32_t fs = ((w ^ sR ^ x) - kNib1) & kGuard;
-  const uint32_t fp = ((w ^ spR ^ x) - kNib1) & kGuard;
-  const uint32_t idx = (uint32_t)__popc(fs) * 9u + (uint32_t)__popc(fp);
-  const uint2 row = Tb.rows[idx];
-  const bool accept = CMP64 ? ((unsigned long long)u < Tb.T64[idx]) : (u <= row.x);
+// Metropolis update of arm ARM of a cell (Sec. II.C, Eq. H) with draw u and
+// proposal offset k.  w2 holds the cell's word (sigma_b in nibble b) in both
+// halves, p2 the partner values (arm a^1 of the neighbour in direction a, in
+// nibble a) in both halves.  With the partner in the nibble of the arm itself,
+// the low half is compared with sigma and the high half with sigma' at once: a
+// low nibble of x ^ prop is y = nibble ^ sigma and y + 7 has bit 3 set iff it
+// differs; a high one is 7 ^ y for sigma', and (7 ^ y) + 1 has bit 3 set iff it
+// is equal (no carry leaves a nibble).  For an arm b != a the two bits add up
+// to 1 + [sigma_b = sigma'] - [sigma_b = sigma], its part of dN_sigma plus 1;
+// for the partner they add up to dN_HB + 1.  dp4a adds both bytes of a pair of
+// arms with the same weight: 1 for the pair that holds ARM, 4 for the other, so
+// an even nibble's bits (8 in their byte) go to the two-bit sums at bits 3 and
+// 5, an odd one's (128) to those at bits 7 and 9 -- the byte offset of a pair
+// of words, on top of the lane's copy.  One compare of eight nibbles and one
+// dp4a take the place of a compare and a population count for sigma and for
+// sigma' each (169 -> 143 thread instructions a cell, ALU 73 -> 61 operations,
+// shared-memory wavefronts 38 -> 36): 4096^2 89.4 against 104.1 us per step,
+// 256 mixed replicas 109.8 against 151.5 (97.4 and 140.6 before the second
+// copy of the rows and the folded complement).
+template <bool CMP64, int ARM>
+__device__ __forceinline__ uint32_t update_arm2(uint32_t w2, uint32_t p2, uint32_t u, uint32_t k,
+                                                uint32_t q, const Tables2& Tb, uint32_t& pk) {
+  // 4 sigma: the byte offset of sigma's entries
+  const uint32_t s4 = ((ARM == 0) ? (w2 << 2) : (w2 >> (4 * ARM - 2))) & 0x1Cu;
+  const uint32_t e = k * (4u * q) + s4;
+  const uint32_t vR = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(Tb.prop) + e);
+  const uint32_t nR = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(Tb.next) + e);
+  constexpr uint32_t mask = 0x000F000Fu << (4 * ARM);
+  const uint32_t x = (w2 & ~mask) | (p2 & mask);
+  const uint32_t f = ((x ^ vR) + 0x11117777u) & 0x88888888u;
+  const uint32_t copy = (threadIdx.x & 1u) * (uint32_t)(4 * kRowCopy);
+  const char* row = reinterpret_cast<const char*>(Tb.rows + (ARM & 1) * kRowWords) +
+                    __dp4a(f, (ARM < 2) ? 0x04010401u : 0x01040104u, copy);
+  const uint32_t thr = *reinterpret_cast<const uint32_t*>(row);
+  const uint32_t change = *reinterpret_cast<const uint32_t*>(row + 4);
+  bool accept = u <= thr;
+  if (CMP64) accept = accept && change != 0u;
   if (accept) {
-    const uint32_t mask = 0xFu << (4u * a);
-    w = (w & ~mask) | (spR & mask);
-    pk += row.y;
+    w2 = (w2 & ~mask) | (nR & mask);
+    pk += change;
   }
-  return w;
+  return w2;
 }
 
 // Count word of a cell: nibble v = number of its arms in state v.
@@ -185,34 +194,28 @@ __device__ __forceinline__ uint32_t update_in_word(uint32_t own, uint32_t xm_wor
                                                    const KEYS& keys, uint32_t q,
                                                    const Tables2& Tb, uint32_t& pk,
                                                    uint32_t* s_hist4) {
-  // partner operands: arm 0 (+x) <-> arm 1 of the +x cell, arm 1 (-x) <->
-  // arm 0 of the -x cell, arm 2 (+y) <-> arm 3 of the +y cell, arm 3 (-y)
-  // <-> arm 2 of the -y cell; each partner value, masked where it lies,
-  // is copied into nibbles 4..7 by one multiply-add that also sets the
-  // guard bits (the multiplier moves it there from its own nibble)
-  const int hi = (HI >= 0) ? HI : hi_rt;
-  uint32_t w, x0, x1, x2, x3;
-  if (hi) {
-    w = own >> 16;
-    x0 = (xp_word & 0x70u) * 0x1111000u + kGuard;           // nibble 1 of the +x word
-    x1 = (own & 0x7u) * 0x11110000u + kGuard;               // nibble 0 of the own word
-    x2 = ((yp_word >> 12) & 0x70000u) * 0x1111u + kGuard;   // nibble 7 of the +y word
-    x3 = ((ym_word >> 8) & 0x70000u) * 0x1111u + kGuard;    // nibble 6 of the -y word
-  } else {
-    w = own & 0xFFFFu;
-    x0 = ((own >> 4) & 0x70000u) * 0x1111u + kGuard;        // nibble 5 of the own word
-    x1 = (xm_word & 0x70000u) * 0x1111u + kGuard;           // nibble 4 of the -x word
-    x2 = (yp_word & 0x7000u) * 0x11110u + kGuard;           // nibble 3 of the +y word
-    x3 = (ym_word & 0x700u) * 0x111100u + kGuard;           // nibble 2 of the -y word
-  }
+  // partners: arm 0 (+x) <-> arm 1 of the +x cell, arm 1 (-x) <-> arm 0 of
+  // the -x cell, arm 2 (+y) <-> arm 3 of the +y cell, arm 3 (-y) <-> arm 2 of
+  // the -y cell.  Each lies in the byte it has to go to or a whole byte
+  // away, in the other nibble: the even arms' partners are gathered in the
+  // odd nibbles of A (both halves alike), the odd arms' in the even nibbles of
+  // B, and the two are shifted past each other.
+  const bool hi = ((HI >= 0) ? HI : hi_rt) != 0;
+  // hi: byte 0 of the +x word / the own word, byte 3 of the +y / -y word;
+  // low half: byte 2 of the own word / the -x word, byte 1 of the +y / -y word
+  const uint32_t sel = hi ? 0x7070u : 0x5252u;
+  const uint32_t A = __byte_perm(hi ? xp_word : own, yp_word, sel);
+  const uint32_t B = __byte_perm(hi ? own : xm_word, ym_word, sel);
+  const uint32_t p2 = ((A >> 4) & 0x0F0F0F0Fu) | ((B << 4) & 0xF0F0F0F0u);
+  uint32_t w = twice(own, hi);
   uint32_t acc[4], kk[4];
   draws<RNG_WORDS>(c, s_lo, s_hi, keys, q, acc, kk);
-  w = update_arm2<CMP64, 0>(w, x0, acc[0], kk[0], 0u, Tb, pk);
-  w = update_arm2<CMP64, 1>(w, x1, acc[1], kk[1], 1u, Tb, pk);
-  w = update_arm2<CMP64, 2>(w, x2, acc[2], kk[2], 2u, Tb, pk);
-  w = update_arm2<CMP64, 3>(w, x3, acc[3], kk[3], 3u, Tb, pk);
+  w = update_arm2<CMP64, 0>(w, p2, acc[0], kk[0], q, Tb, pk);
+  w = update_arm2<CMP64, 1>(w, p2, acc[1], kk[1], q, Tb, pk);
+  w = update_arm2<CMP64, 2>(w, p2, acc[2], kk[2], q, Tb, pk);
+  w = update_arm2<CMP64, 3>(w, p2, acc[3], kk[3], q, Tb, pk);
   if (s_hist4) hist_add_cell(s_hist4, count_word4(w));
-  return hi ? ((own & 0xFFFFu) | (w << 16)) : ((own & 0xFFFF0000u) | w);
+  return __byte_perm(own, w, hi ? 0x5410u : 0x3254u);
 }
 
 // Staged input: rows y0-2 .. y0+TR+1 and words p0-4 .. p0+TW+3 (a 16-byte
@@ -472,10 +475,9 @@ __device__ __forceinline__ void colour1(const StepView<KEYS>& v, const TileGeom&
 // colour-1 update reads only the colour-0 halves of its neighbours, which
 // colour 1 does not change), and the tile is copied out with 16-byte loads
 // and stores.  PAIRS: row pairs per loop iteration (the compiler's unroll
-// factor; 2 where the kernel has the registers for it: the wavefront sweep
-// at 64 registers, 4096^2 103.0 against 104.8 us per step; the tiled sweep at
-// 48 registers keeps 1, where 2 spilled 76 bytes and ran at 563 against 583
-// sigma-updates/ns).
+// factor): the wavefront sweep 4 (4096^2 87.5 against 89.4 us per step with 2,
+// 91.1 with 1 or with all 8), the batched kernel 2 (256 mixed replicas 108.2
+// against 109.7 with 1, 110.4 with 4), the tiled sweep 1 (2 changed nothing).
 // ---------------------------------------------------------------------------
 template <int RNG_WORDS, bool CMP64, int TR, int TW, int NT, bool REC, int PAIRS,
           typename KEYS>

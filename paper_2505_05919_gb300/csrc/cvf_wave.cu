@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(kThreads, kWaveBlocksPerSM)
     const int r = s_r, t = s_t, g = s_g, staged = s_staged;
     const long long step = step0 + r;
     if (g != g_cur) {  // block-uniform
-      fill_rows2(Tb, A.table24, g);
+      fill_rows2(Tb, A.table24, g, kThreads);
       g_cur = g;
     }
     StepView<KeysStep> v;
@@ -371,9 +371,9 @@ __global__ void __launch_bounds__(kThreads, kWaveBlocksPerSM)
     const bool rec = step_recorded(every, step);
     if constexpr (WALK) {
       if (rec)
-        colour0_walk<RNG_WORDS, CMP64, TR, TW, kThreads, true, 2>(v, gm, S, Tb, cnt, s_hist4);
+        colour0_walk<RNG_WORDS, CMP64, TR, TW, kThreads, true, 4>(v, gm, S, Tb, cnt, s_hist4);
       else
-        colour0_walk<RNG_WORDS, CMP64, TR, TW, kThreads, false, 2>(v, gm, S, Tb, cnt, nullptr);
+        colour0_walk<RNG_WORDS, CMP64, TR, TW, kThreads, false, 4>(v, gm, S, Tb, cnt, nullptr);
     } else {
       colour0<RNG_WORDS, CMP64, TR, TW, kThreads, kWaveShape>(v, gm, S, Tb, cnt,
                                                                rec ? s_hist4 : nullptr);
@@ -438,9 +438,9 @@ __global__ void __launch_bounds__(kThreads, kWaveBlocksPerSM)
     }
     if constexpr (WALK) {
       if (rec)
-        colour1_walk<RNG_WORDS, CMP64, TR, TW, kThreads, true, 2>(v, gm, S, Tb, cnt, s_hist4);
+        colour1_walk<RNG_WORDS, CMP64, TR, TW, kThreads, true, 4>(v, gm, S, Tb, cnt, s_hist4);
       else
-        colour1_walk<RNG_WORDS, CMP64, TR, TW, kThreads, false, 2>(v, gm, S, Tb, cnt, nullptr);
+        colour1_walk<RNG_WORDS, CMP64, TR, TW, kThreads, false, 4>(v, gm, S, Tb, cnt, nullptr);
     } else {
       colour1<RNG_WORDS, CMP64, TR, TW, kThreads, kWaveShape>(v, gm, S, Tb, cnt,
                                                                rec ? s_hist4 : nullptr);
