@@ -86,7 +86,8 @@ class Lattice3:
 
     def set_resident(self, mode: int) -> None:
         """1: the cube resident in one thread-block cluster during each call
-        (L a multiple of 8, 16 <= L <= 64); 0: four launches per step; -1: choose."""
+        (L a multiple of 8, 16 <= L <= 64); 0: from global memory; -1: choose
+        (cvf3_set_resident in cvf.h)."""
         _capi.cvf3_set_resident(self.h, mode)
 
     def resident(self) -> bool:

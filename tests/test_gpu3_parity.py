@@ -326,3 +326,50 @@ def test_lattice3_eta_every_step(T, P, init):
             assert np.array_equal(lat.eta(), ref.eta())
         assert np.array_equal(lat.state(), ref.state())
     assert ref.acc_eta > 0
+
+
+# The dataflow sweep at its edges: blocks whose last warp is partly empty, the
+# last side with one group per thread and the first with several (51 / 52), rows
+# that groups cross (L % 4 != 0) with and without eta moves, one block, the
+# 64-bit compare, gate flips, every step recorded.
+FLOW = [
+    (2, 1, 60, 1, {}),
+    (10, 1, 30, 1, dict(q=2)),
+    (16, 1, 40, 1, dict(q=8)),
+    (32, 1, 12, 3, dict(init=oracle.INIT_ORDERED)),
+    (33, 0, 12, 1, {}),
+    (34, 1, 12, 4, dict(kT=1e-3)),
+    (44, 1, 8, 1, {}),
+    (51, 0, 6, 2, {}),
+    (52, 1, 6, 1, {}),
+    (54, 1, 5, 0, dict(q=3)),
+    (61, 0, 4, 1, dict(kT=1e-3)),
+    (12, 1, 300, 1, dict(gates=True)),
+    (33, 0, 120, 1, dict(gates=True)),
+]
+
+
+@pytest.mark.parametrize("L,eta,steps,every,extra", FLOW, ids=["L%d-%d" % (c[0], i) for i, c in enumerate(FLOW)])
+def test_lattice3_dataflow_sweep(L, eta, steps, every, extra):
+    extra = dict(extra)
+    if extra.pop("gates", False):
+        op = oracle.params3(L=L, seed=700 + L, kT=1.0, P=0.5, J=0.0, v_HB=0.0, epsilon=0.0,
+                            v_iso_init=1.98, dv_max_frac=0.02, eta_moves=eta)
+    elif "kT" in extra:
+        op = oracle.params3(L=L, seed=700 + L, eta_moves=eta, **extra)
+    else:
+        op = oracle.physical_params3(300.0, 0.1, L=L, seed=700 + L, dv_max_frac=0.05, eta_moves=eta, **extra)
+    ref = oracle.Oracle3(op)
+    want = ref.run(steps, every)
+    with Lattice3(params_from_dict(asdict(op))) as lat:
+        lat.sweep(steps // 3, every)
+        lat.sweep(steps - steps // 3, every)
+        got, overflow = lat.drain()
+        s, o, eta_got, recount = lat.state(), lat.observables(), lat.eta(), lat.recount()
+    assert not overflow and len(got) == len(want)
+    assert np.array_equal(s, ref.state())
+    assert np.array_equal(eta_got, ref.eta())
+    _same(o, ref.observables(), L)
+    assert recount == (o["n_hb_raw"], o["n_coop"])
+    for i, (g, w) in enumerate(zip(got, want)):
+        _same(g, w, ("record", i))
