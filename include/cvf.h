@@ -203,11 +203,15 @@ int cvf_state_device_ptr(cvf_handle *h, void **dev_ptr);
  * 2 swept by one persistent cooperative launch per call in which a tile of
  * step s + 1 waits only for the tiles around it to finish step s (a
  * wavefront; the volume moves decided ahead by one block; L a multiple of 8
- * and at least 3 x 3 tiles); -1 = automatic (chosen at creation: the
- * resident form for small lattices, else the largest tile shape whose tiles
- * fill every resident block, swept as a wavefront from L = 256 up).  The result does not depend on the config;
- * set_tiles waits for the stream.  CVF_EINVAL for other values, or a config
- * that does not apply to the lattice. */
+ * and at least 3 x 3 tiles); -1 = automatic (chosen at creation): a lattice
+ * small enough (about L <= 1094 on 152 SMs) has no tiles and runs as one
+ * persistent launch per call in which every word carries its own progress;
+ * get_tiles then still names the configuration of the rule for larger ones --
+ * the resident form for small lattices, else the largest tile shape whose tiles
+ * fill every resident block, swept as a wavefront from L = 256 up -- and the
+ * larger ones run it.  The layered schedule has no tiles.  The result does not
+ * depend on the config; set_tiles waits for the stream.  CVF_EINVAL for other
+ * values, or a config that does not apply to the lattice. */
 int cvf_set_tiles(cvf_handle *h, int32_t config);
 int cvf_get_tiles(cvf_handle *h, int32_t *config, int32_t *rows,
                   int32_t *words);

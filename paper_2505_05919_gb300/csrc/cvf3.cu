@@ -991,8 +991,7 @@ struct cvf3_handle {
   int res_ctas;   // CTAs of that cluster (0 until it is first needed)
   bool flow;        // the dataflow sweep, where no cluster was asked for
   Flow3Plan plan;
-  WaveHdr* wave;    // its scratch and its tagged copy of the cube
-  uint32_t* copy;
+  WaveHdr* wave;    // its scratch and, behind it, its tagged copy of the cube
   int grid;
   int grid_count;
   int grid_eta;
@@ -1005,7 +1004,6 @@ void release3(cvf3_handle* h) {
   if (!h) return;
   if (h->graph) cudaGraphExecDestroy(h->graph);
   if (h->wave) cudaFree(h->wave);
-  if (h->copy) cudaFree(h->copy);
   if (h->own_state && h->state) cudaFree(h->state);
   if (h->ctrl) cudaFree(h->ctrl);
   if (h->ring) cudaFree(h->ring);
@@ -1046,6 +1044,8 @@ void enqueue_step3(cvf3_handle* h, cudaStream_t s) {
 int build_graph3(cvf3_handle* h) {
   if (h->graph) return CVF_OK;
   cudaGraph_t g = nullptr;
+  if (!h->cap_stream)
+    CVF_CUDA_CHECK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   CVF_CUDA_CHECK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
   for (int i = 0; i < kGraphSteps3; ++i) enqueue_step3(h, h->cap_stream);
   cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
@@ -1128,7 +1128,6 @@ int cvf3_create(const cvf_params* p, void* stream, void* dev_state, cvf3_handle*
       return code_;                                                               \
     }                                                                             \
   } while (0)
-  CREATE_CHECK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   if (dev_state) {
     h->state = reinterpret_cast<uint32_t*>(dev_state);
     h->own_state = false;
@@ -1201,13 +1200,17 @@ int cvf3_create(const cvf_params* p, void* stream, void* dev_state, cvf3_handle*
   h->resident = resident3_auto(A, h->cmp64);
   h->plan = flow3_plan(A, h->cmp64);
   h->flow = h->plan.blocks > 0 && A.groups <= kFlowMaxGroups;
-  h->cluster = h->resident && !h->flow;
   if (h->flow) {
-    const size_t bytes = sizeof(uint32_t) * h->plan.copy_words;
-    CREATE_CHECK(cudaMalloc(reinterpret_cast<void**>(&h->wave), sizeof(WaveHdr)));
-    CREATE_CHECK(cudaMalloc(reinterpret_cast<void**>(&h->copy), bytes));
-    CREATE_CHECK(cudaMemsetAsync(h->copy, 0, bytes, h->stream));
+    const size_t bytes = sizeof(WaveHdr) + sizeof(uint32_t) * h->plan.copy_words;
+    if (cudaMalloc(reinterpret_cast<void**>(&h->wave), bytes) != cudaSuccess) {
+      cudaGetLastError();  // no room for the copy: the cube runs without it
+      h->wave = nullptr;
+      h->flow = false;
+    } else {
+      CREATE_CHECK(cudaMemsetAsync(h->wave, 0, bytes, h->stream));
+    }
   }
+  h->cluster = h->resident && !h->flow;
   h->grid_count = (int)std::max<long long>(
       1, std::min<long long>((h->N + kThreads3 - 1) / kThreads3, (long long)sm_count() * 8));
   h->grid_eta = (int)std::max<long long>(
@@ -1251,8 +1254,7 @@ int cvf3_sweep(cvf3_handle* h, int64_t n_sweeps, int32_t record_every) {
       const long long n = std::min<long long>(chunk, n_sweeps - done);
       CVF_CUDA_CHECK(h->cluster ? launch_resident3(h->args, h->cmp64, h->res_ctas, n, record_every,
                                                    h->stream)
-                                : launch_flow3(h->args, h->plan, h->wave, h->copy, n, record_every,
-                                               h->stream));
+                                : launch_flow3(h->args, h->plan, h->wave, n, record_every, h->stream));
     }
     return CVF_OK;
   }

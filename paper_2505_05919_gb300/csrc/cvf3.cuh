@@ -57,9 +57,10 @@ struct Flow3Plan {
   size_t copy_words;
 };
 Flow3Plan flow3_plan(const Args3& A, bool cmp64);
-// Enqueues the call's steps in one cooperative launch; H is its scratch.
-cudaError_t launch_flow3(const Args3& A, const Flow3Plan& P, WaveHdr* H, uint32_t* copy,
-                         long long n_steps, int every, cudaStream_t s);
+// Enqueues the call's steps in one cooperative launch; H is its scratch, and the
+// copy lies behind it.
+cudaError_t launch_flow3(const Args3& A, const Flow3Plan& P, WaveHdr* H, long long n_steps,
+                         int every, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Arm order and segments of a step.  The order is permutation number

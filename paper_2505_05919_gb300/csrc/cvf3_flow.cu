@@ -26,9 +26,9 @@
 // The threads of a block share the step's plan, its gate and its counts
 // through a ring of kWaveRing steps in shared memory, kept by one more warp
 // (the clerk): it makes the plans, waits for the volume moves that block 0
-// decides ahead (wave_engine), gathers the counts of the block's warps and
-// commits the steps it completes (wave_commit).  So no warp that sweeps waits
-// for anything but the words it reads.
+// decides ahead (wave_engine) and gathers the counts of the block's warps; a
+// warp of block 0 commits the steps (flow_commit).  So no warp that sweeps
+// waits for anything but the words it reads.
 //
 // All blocks are co-resident (a cooperative launch) and a part waits only for
 // earlier parts, so the earliest unfinished part can always run.  Every wait is
@@ -43,11 +43,11 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <cstring>
+#include <climits>
 
 #include "cvf3.cuh"
+#include "cvf_flow.cuh"
 #include "cvf_host.h"
-#include "cvf_wave.cuh"
 
 namespace cvf {
 namespace {
@@ -61,18 +61,6 @@ namespace {
 constexpr int kFlowThreadsOne = 224, kFlowThreadsMany = 480;
 inline int flow_threads(bool one) { return one ? kFlowThreadsOne : kFlowThreadsMany; }
 constexpr int kFlowHead = 32;                    // words before the copy's cells (word 0: the tag)
-constexpr unsigned int kFlowSpinLimit = 1u << 21;  // loads of L2: about a second
-
-// The ring of steps a block's warps share.
-struct FlowSlot {
-  unsigned long long plan;
-  int g;
-  int ready;             // relative step + 1 once plan and gate are set
-  int hb, pairs, moves;  // counts of the warps that finished the step
-  int done;              // their number
-  uint32_t hist[8];
-};
-
 struct FlowSmem {
   Tables3 Tb[2];  // per gate (the proposals in the first)
   unsigned long long eta_thr[2][9];
@@ -80,117 +68,6 @@ struct FlowSmem {
   uint32_t forbid[8][9];  // eta copies that are 0 at corner j in configuration c
   FlowSlot ring[kWaveRing];
 };
-
-__device__ __forceinline__ uint4 ld_flow4(const uint32_t* p) {
-  uint4 v;
-  asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p)
-               : "memory");
-  return v;
-}
-__device__ __forceinline__ uint32_t ld_flow(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_flow4(uint32_t* p, uint4 v) {
-  asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x),
-               "r"(v.y), "r"(v.z), "r"(v.w)
-               : "memory");
-}
-__device__ __forceinline__ void st_flow(uint32_t* p, uint32_t v) {
-  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Bit 31 set iff the word's tag is behind the one needed (`need` in bits
-// 24..31, the bits below clear).
-__device__ __forceinline__ uint32_t behind(uint32_t w, uint32_t need) { return w - need; }
-
-// After a warp's `spins` unsuccessful polls (all 32 lanes): true when it has to
-// stop, since another wait gave up or this one does.
-__device__ __noinline__ bool flow_stop(unsigned int spins, WaveHdr* H, unsigned int* err) {
-  const bool stop = *(volatile unsigned int*)&H->abort != 0u;
-  if (__any_sync(0xFFFFFFFFu, stop)) return true;
-  if (spins < kFlowSpinLimit) return false;
-  if ((threadIdx.x & 31u) == 0u) {
-    atomicOr(err, 1u);
-    atomicExch(&H->abort, 1u);
-  }
-  return true;
-}
-
-// The clerk (one thread): keeps the ring, gathers the counts and commits.
-__device__ void flow_clerk(const Args3& A, FlowSlot* ring, int warps, int blocks, WaveHdr* H,
-                           uint32_t* copy, uint32_t end_tag, long long step0, long long n_steps,
-                           int every) {
-  Ctrl* const ctl = A.ctrl;
-  long long ready = 0, flush = 0, commit = -1;  // next steps; the one to commit
-  unsigned int idle = 0;
-  while (flush < n_steps || commit >= 0) {
-    bool moved = false;
-    if (ready < n_steps) {
-      const WaveMove& m = H->vring[ready % kWaveRing];
-      if (ld_acquire(&m.tag) >= (unsigned int)(ready + 1) &&
-          (ready < kWaveRing ||
-           ld_acquire(&H->committed) >= (unsigned int)(ready - kWaveRing + 1))) {
-        FlowSlot& s = ring[ready % kWaveRing];
-        s.g = *(volatile const int*)&m.g;
-        s.plan = make_plan(step0 + ready, A.keys);
-        __threadfence_block();
-        *(volatile int*)&s.ready = (int)(ready + 1);
-        ++ready;
-        moved = true;
-      }
-    }
-    if (commit < 0 && flush < n_steps) {
-      FlowSlot& s = ring[flush % kWaveRing];
-      if (*(volatile int*)&s.done == warps) {
-        __threadfence_block();
-        volatile FlowSlot* v = &s;
-        WaveAcc* const slot = &H->acc[flush % kWaveRing];
-        atomicAdd(&slot->hb, (unsigned long long)(long long)v->hb);
-        atomicAdd(&slot->pairs, (unsigned long long)(long long)v->pairs);
-        atomicAdd(&slot->moves, (unsigned long long)(long long)v->moves);
-        if (step_recorded(every, step0 + flush)) {
-          for (int k = 0; k < 8; ++k) {
-            if (v->hist[k]) atomicAdd(&slot->hist[k], (unsigned long long)v->hist[k]);
-            v->hist[k] = 0;
-          }
-        }
-        v->hb = v->pairs = v->moves = v->done = 0;
-        // the counts before the completion count; who completes the step
-        // commits it (its fence acquires every other block's counts)
-        fence_acq_rel_gpu();
-        if (atom_add_relaxed_u32(&slot->done, 1u) + 1u == (unsigned int)blocks) {
-          fence_acq_rel_gpu();
-          commit = flush;
-        }
-        ++flush;
-        moved = true;
-      }
-    }
-    if (commit >= 0 && (commit == 0 || ld_acquire(&H->committed) >= (unsigned int)commit)) {
-      // every block has finished the call's last step (and read the tag it
-      // started from): the tag the next call starts from
-      if (commit == n_steps - 1) copy[0] = end_tag;
-      wave_commit(ctl, *A.vol, A.ring, A.ring_cap, every, H, step0, commit);
-      commit = -1;
-      moved = true;
-    }
-    if (moved) {
-      idle = 0;
-    } else {
-      if (*(volatile unsigned int*)&H->abort) return;
-      if (++idle > kWaitPollLimit) {
-        atomicOr(&ctl->error, 1u);
-        atomicExch(&H->abort, 1u);
-        return;
-      }
-      __nanosleep(64);
-    }
-  }
-}
 
 // ALIGNED: L % 4 == 0, a group (four consecutive cells) lies in one row and
 // its words and its y and z neighbours' are 16-byte vectors; otherwise every
@@ -210,16 +87,15 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
   // block has taken part in the first (last) step
   const long long step0 = *(volatile long long*)&ctl->sweep;
   const uint32_t tag0 = *(volatile uint32_t*)copy + 8u;
+  const uint32_t end_tag = tag0 + 8u * (uint32_t)((unsigned long long)n_steps & 0xFFFFFFu);
   if (blockIdx.x == 0) {
-    stage_volume_args(&U.vol, A.vol);
-    __syncthreads();
-    if (threadIdx.x < 64) wave_engine(ctl, U.vol, A.keys, H, step0, n_steps);
+    flow_books(A, U.vol, H, (int)gridDim.x - 1, copy, end_tag, step0, n_steps, every);
     return;
   }
   constexpr int kFlowThreads = ONE ? kFlowThreadsOne : kFlowThreadsMany;
   constexpr int kFlowBlock = kFlowThreads + 32;
   FlowSmem& S = U.sweep;
-  const uint32_t b = blockIdx.x - 1u, blocks = gridDim.x - 1u;
+  const uint32_t b = blockIdx.x - 1u;
   uint32_t* const F = copy + kFlowHead;             // the cells' words
   uint32_t* const C = F + 4u * (size_t)A.groups;    // the cubes' words
   const uint32_t g_lo = b * groups_per_block, g_hi = min(g_lo + groups_per_block, A.groups);
@@ -251,10 +127,8 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
   }
   __syncthreads();
   if (threadIdx.x >= kFlowThreads) {
-    if (threadIdx.x == kFlowThreads)
-      flow_clerk(A, S.ring, warps, (int)blocks, H, copy,
-                 tag0 + 8u * (uint32_t)((unsigned long long)n_steps & 0xFFFFFFu), step0, n_steps,
-                 every);
+    flow_clerk([&](long long s) { return make_plan(s, A.keys); }, S.ring, warps, H, err, step0,
+               n_steps, every);
     return;
   }
   if ((int)(threadIdx.x >> 5) >= warps) return;
@@ -539,17 +413,7 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
       if (!alive) return;
     }
 
-    const int a1 = __reduce_add_sync(full, (int)(hb_b - nacc + eta_dhb));
-    const int a2 = __reduce_add_sync(full, (int)(dc_b - 5u * nacc));
-    const int a3 = __reduce_add_sync(full, (int)nacc);
-    if ((threadIdx.x & 31u) == 0u) {
-      atomicAdd(&slot.hb, a1);
-      atomicAdd(&slot.pairs, a2);
-      atomicAdd(&slot.moves, a3);
-    }
-    __threadfence_block();
-    __syncwarp();
-    if ((threadIdx.x & 31u) == 0u) atomicAdd(&slot.done, 1);
+    flow_report(slot, (int)(hb_b - nacc + eta_dhb), (int)(dc_b - 5u * nacc), (int)nacc);
   }
 }
 
@@ -558,17 +422,6 @@ const void* flow3_kernel(bool aligned, bool cmp64) {
   if (aligned)
     return cmp64 ? (const void*)k_flow3<true, true, ONE> : (const void*)k_flow3<true, false, ONE>;
   return cmp64 ? (const void*)k_flow3<false, true, ONE> : (const void*)k_flow3<false, false, ONE>;
-}
-
-int resident_blocks(const void* fn, bool one) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, flow_threads(one) + 32, 0) !=
-          cudaSuccess ||
-      per_sm < 1) {
-    cudaGetLastError();
-    return 0;
-  }
-  return per_sm * sm_count();
 }
 
 }  // namespace
@@ -584,7 +437,7 @@ Flow3Plan flow3_plan(const Args3& A, bool cmp64) {
     P.kernel = one ? flow3_kernel<true>(aligned, cmp64) : flow3_kernel<false>(aligned, cmp64);
     P.threads = flow_threads(one) + 32;
     const long long room =
-        (one ? std::min(sm_count(), resident_blocks(P.kernel, one)) : resident_blocks(P.kernel, one)) - 1;
+        std::min(one ? sm_count() : INT_MAX, flow_resident_blocks(P.kernel, P.threads)) - 1;
     if (room < 1 || (one && groups > room * flow_threads(true))) continue;
     const long long share = (groups + room - 1) / room;
     P.groups_per_block = (uint32_t)((share + 31) / 32 * 32);
@@ -594,12 +447,13 @@ Flow3Plan flow3_plan(const Args3& A, bool cmp64) {
   return P;
 }
 
-cudaError_t launch_flow3(const Args3& A, const Flow3Plan& P, WaveHdr* H, uint32_t* copy,
-                         long long n_steps, int every, cudaStream_t s) {
+cudaError_t launch_flow3(const Args3& A, const Flow3Plan& P, WaveHdr* H, long long n_steps,
+                         int every, cudaStream_t s) {
   if (P.blocks < 1) return cudaErrorCooperativeLaunchTooLarge;
   const cudaError_t e = cudaMemsetAsync(H, 0, sizeof(WaveHdr), s);
   if (e != cudaSuccess) return e;
   uint32_t gpb = P.groups_per_block;
+  uint32_t* copy = reinterpret_cast<uint32_t*>(H + 1);
   void* args[6] = {const_cast<Args3*>(&A), &gpb, &H, &copy, &n_steps, &every};
   return cudaLaunchCooperativeKernel(P.kernel, dim3(P.blocks + 1), dim3(P.threads), args, 0, s);
 }

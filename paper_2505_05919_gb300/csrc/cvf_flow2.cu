@@ -1,0 +1,539 @@
+// cvf_flow2.cu -- the MC steps of one square lattice as a single persistent,
+// cooperative launch per call in which every word carries its own progress
+// (dataflow; cvf3_flow.cu is the cubic one and says why it is sound).
+//
+// Checkerboard (k_flow2).  A thread owns V vertically adjacent words (two cells
+// each, one of either colour) of a strip of V rows, in registers for the whole
+// call, and writes them to a copy of the lattice after every colour.  The spare
+// bits 3 and 7 of a cell there hold the number of steps it has finished, modulo
+// 4.  A colour-0 cell of step r needs its four neighbours after r steps, a
+// colour-1 cell after r + 1, and since the neighbours wait for it in turn, they
+// have never done more: a thread loads the words its colour reads until the
+// two bits say so.  Nothing it overwrites is still needed, for the same reason.
+// A call first writes the lattice into the copy with the next number after the
+// one the last call ended with (word 0 of the copy), so no cell of it can be
+// taken for a later one; the words after the last step go to the lattice.
+//
+// Layered schedule (k_flow2_layer).  As the cubic sweep: a segment of the arm
+// order at a time (layer_plan), one 32-bit word per cell in the copy with a
+// 16-bit count of finished parts above the cell, four cells of a row per thread
+// and group.
+//
+// What bounds them: the chain of a part -- store, the neighbour's load of it
+// (0.27 to 0.5 us between SMs), the four arm updates -- up to about 512^2, the
+// instructions of the cells beyond (the launches and waits that it replaces
+// took 2.7 us per step at 64^2, 8.2 at 258^2, 7.3 at 512^2 and 11.9 at 1024^2;
+// now 1.8, 1.9, 2.7 and 7.6).  The draws of a part are made before its first
+// load.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "cvf_fastdiv.cuh"
+#include "cvf_flow.cuh"
+#include "cvf_flow2.cuh"
+#include "cvf_host.h"
+#include "cvf_lattice.cuh"
+#include "cvf_tile.cuh"
+
+namespace cvf {
+namespace {
+
+constexpr int kFlow2Head = 32;  // words before the copy's cells (word 0: the tag)
+
+// Tables of both gates and the ring of steps.
+struct Flow2Smem {
+  Tables2 Tb[2];
+  FlowSlot ring[kWaveRing];
+};
+
+template <typename SMEM>
+__device__ __forceinline__ void flow2_setup(SMEM& S, const LatticeArgs& A, int threads) {
+  for (int g = 0; g < 2; ++g) {
+    fill_rows2(S.Tb[g], A.table24, g, threads);
+    fill_prop2(S.Tb[g], A.q);
+  }
+  uint32_t* ring = reinterpret_cast<uint32_t*>(S.ring);
+  for (int i = threadIdx.x; i < (int)(sizeof(S.ring) / 4); i += threads) ring[i] = 0u;
+}
+
+// Waits (a whole warp) until the clerk has step rel ready; false to stop.
+__device__ __forceinline__ bool flow_ready(const FlowSlot& slot, long long rel, WaveHdr* H,
+                                           unsigned int* err) {
+  unsigned int spins = 0;
+  while (!__all_sync(0xFFFFFFFFu, *(const volatile int*)&slot.ready == (int)(rel + 1))) {
+    if ((++spins & 1023u) == 0u && flow_stop(spins >> 6, H, err)) return false;
+  }
+  __threadfence_block();
+  return true;
+}
+
+// A warp's counts of a step (and N_q' in the 16-bit lanes v, v + 4 of h[v])
+// into its slot.
+__device__ __forceinline__ void flow_report2(FlowSlot& slot, const TileCounts& cnt, bool rec,
+                                             const uint32_t h[4]) {
+  if (rec) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const uint32_t lanes = __reduce_add_sync(0xFFFFFFFFu, h[v]);
+      if ((threadIdx.x & 31u) == 0u) {
+        if (lanes & 0xFFFFu) atomicAdd(&slot.hist[v], lanes & 0xFFFFu);
+        if (lanes >> 16) atomicAdd(&slot.hist[v + 4], lanes >> 16);
+      }
+    }
+  }
+  flow_report(slot, cnt.dhb(), cnt.dc(), (int)cnt.nacc);
+}
+
+// The two spare bits of both cells of a word for t finished steps (of the low
+// cell, the high cell).
+__device__ __forceinline__ uint32_t tag_bits(uint32_t t_low, uint32_t t_high) {
+  return ((t_low & 1u) << 3) | ((t_low & 2u) << 6) | ((t_high & 1u) << 19) | ((t_high & 2u) << 22);
+}
+
+// The Philox words of a cell's draws, before they are split.
+template <int RNG_WORDS>
+struct CellWords {
+  Words4 u, p;  // p: two words per update only
+};
+template <int RNG_WORDS>
+__device__ __forceinline__ CellWords<RNG_WORDS> cell_words(uint32_t c, const StepDraw& sd,
+                                                           const RoundKeys& K) {
+  CellWords<RNG_WORDS> w;
+  w.u = philox_cell(c, sd.acc, K);
+  w.p = (RNG_WORDS == 2) ? philox_cell(c, sd.prop, K) : w.u;
+  return w;
+}
+
+template <int RNG_WORDS, bool CMP64, int V, int NT>
+__global__ void __launch_bounds__(NT + 32, 1)
+    k_flow2(const __grid_constant__ LatticeArgs A, const __grid_constant__ Flow2Geom G, WaveHdr* H,
+            uint32_t* copy, long long n_steps, int every) {
+  __shared__ union {
+    Flow2Smem sweep;
+    VolumeArgs vol;  // the engine block's copy of the parameters
+  } U;
+  Ctrl* const ctl = A.ctrl;
+  unsigned int* const err = &ctl->error;
+  // the committed step count and the copy's tag: neither changes before every
+  // block has taken part in the first (last) step
+  const long long step0 = *(volatile long long*)&ctl->sweep;
+  const uint32_t tag0 = *(volatile uint32_t*)copy + 1u;
+  if (blockIdx.x == 0) {
+    flow_books(A, U.vol, H, (int)gridDim.x - 1, copy,
+               tag0 + (uint32_t)((unsigned long long)n_steps & 0xFFFFFFu), step0, n_steps, every);
+    return;
+  }
+  Flow2Smem& S = U.sweep;
+  uint32_t* const F = copy + kFlow2Head;
+  const uint32_t t_lo = (blockIdx.x - 1u) * G.per_block, t_hi = min(t_lo + G.per_block, G.items);
+  const int warps = (int)((t_hi - t_lo + 31u) / 32u);
+  flow2_setup(S, A, NT + 32);
+  __syncthreads();
+  if (threadIdx.x >= NT) {
+    flow_clerk([](long long) { return 0ull; }, S.ring, warps, H, err, step0, n_steps, every);
+    return;
+  }
+  if ((int)(threadIdx.x >> 5) >= warps) return;
+  const unsigned int full = 0xFFFFFFFFu;
+  const bool mine = t_lo + threadIdx.x < t_hi;
+  const uint32_t item = min(t_lo + threadIdx.x, t_hi - 1u);  // (a lane without one reads along)
+  const uint32_t L = (uint32_t)A.L, Lh = L >> 1, q = A.q;
+  const uint32_t strip = fdiv(item, G.div_row), p = item - strip * Lh, y0 = strip * (uint32_t)V;
+  const uint32_t h = min((uint32_t)V, L - y0);  // rows (even, but for V = 1)
+  const uint32_t up = ((y0 == 0u) ? L - 1u : y0 - 1u) * Lh + p;
+  const uint32_t down = ((y0 + h == L) ? 0u : y0 + h) * Lh + p;
+  const uint32_t left = (p == 0u) ? Lh - 1u : p - 1u, right = (p + 1u == Lh) ? 0u : p + 1u;
+  const uint32_t odd0 = y0 & 1u;  // 0 unless V = 1
+
+  uint32_t w[V];
+  {
+    const long long N = (long long)L * L;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(A.state + (size_t)(step0 & 1) * N);
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      w[k] = 0u;
+      if ((uint32_t)k < h && dcheck((y0 + k) * Lh + p < L * Lh, err, kSiteStage)) {
+        w[k] = __ldcg(src + (y0 + k) * Lh + p);
+        if (mine) st_flow(F + (y0 + k) * Lh + p, w[k] | tag_bits(tag0, tag0));
+      }
+    }
+  }
+
+  for (long long rel = 0; rel < n_steps; ++rel) {
+    const long long step = step0 + rel;
+    FlowSlot& slot = S.ring[rel % kWaveRing];
+    const uint32_t tag = tag0 + (uint32_t)((unsigned long long)rel & 0xFFFFFFu);
+    const StepDraw sd = step_draw((uint32_t)((unsigned long long)step & 0xFFFFFFFFu),
+                                  (uint32_t)((unsigned long long)step >> 32), A.keys);
+    uint32_t pk = 0;
+    int g = 0;
+#pragma unroll
+    for (int colour = 0; colour < 2; ++colour) {
+      CellWords<RNG_WORDS> draw[V];
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        const uint32_t hi = (odd0 + (uint32_t)(k ^ colour)) & 1u;
+        draw[k] = cell_words<RNG_WORDS>((y0 + k) * L + 2u * p + hi, sd, A.keys);
+      }
+      if (colour == 0) {
+        if (!flow_ready(slot, rel, H, err)) return;
+        g = slot.g;
+      }
+      // what the neighbours' cells (of the other colour) have to show
+      const uint32_t need = tag_bits(tag + (uint32_t)colour, tag + (uint32_t)colour);
+      uint32_t side[V], top = 0u, bottom = 0u;
+      for (unsigned int spins = 0;;) {
+        uint32_t late = 0u;
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+          const uint32_t hi = (odd0 + (uint32_t)(k ^ colour)) & 1u;
+          side[k] = 0u;
+          if ((uint32_t)k < h) {
+            // the low cell's left neighbour is the high cell of the word to the
+            // left, the high cell's right one the low cell to the right
+            side[k] = ld_flow(F + (y0 + k) * Lh + (hi ? right : left));
+            late |= (side[k] ^ need) & (hi ? 0x88u : 0x880000u);
+          }
+        }
+        const uint32_t hi0 = (odd0 + (uint32_t)colour) & 1u;          // row 0's half
+        const uint32_t hi1 = (odd0 + h - 1u + (uint32_t)colour) & 1u;  // the last row's
+        top = ld_flow(F + up);
+        bottom = ld_flow(F + down);
+        late |= (top ^ need) & (hi0 ? 0x880000u : 0x88u);
+        late |= (bottom ^ need) & (hi1 ? 0x880000u : 0x88u);
+        if (__all_sync(full, late == 0u)) break;
+        if ((++spins & 255u) == 0u && flow_stop(spins, H, err)) return;
+      }
+      if (mine) {
+        const Tables2& Tb = S.Tb[g];
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+          if ((uint32_t)k < h) {
+            uint32_t acc[4], kk[4];
+            split_draws<RNG_WORDS>(draw[k].u, draw[k].p, q, acc, kk);
+            const uint32_t ym = (k == 0) ? top : w[(k > 0) ? k - 1 : 0];
+            const uint32_t yp = ((uint32_t)k + 1u == h) ? bottom : w[(k + 1 < V) ? k + 1 : 0];
+            const int hi = (V == 1) ? (int)((odd0 + (uint32_t)colour) & 1u) : ((k ^ colour) & 1);
+            const uint32_t cell =
+                (V == 1) ? update_cell<CMP64>(w[k], side[k], side[k], ym, yp, hi, acc, kk, q, Tb, pk)
+                : hi ? update_cell<CMP64, 1>(w[k], side[k], side[k], ym, yp, 1, acc, kk, q, Tb, pk)
+                     : update_cell<CMP64, 0>(w[k], side[k], side[k], ym, yp, 0, acc, kk, q, Tb, pk);
+            w[k] = put_cell(w[k], cell, hi != 0);
+            const uint32_t other = tag + (uint32_t)colour;  // steps the word's other cell has done
+            st_flow(F + (y0 + k) * Lh + p,
+                    w[k] | (hi ? tag_bits(other, tag + 1u) : tag_bits(tag + 1u, other)));
+          }
+        }
+      }
+    }
+    TileCounts cnt{0, 0, 0};
+    cnt.add(pk);
+    const bool rec = step_recorded(every, step);
+    uint32_t hist[4] = {0u, 0u, 0u, 0u};
+    if (rec && mine) {
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        if ((uint32_t)k < h) {
+          const uint32_t n = count_word4(w[k] & 0xFFFFu) + count_word4(w[k] >> 16);  // nibbles <= 8
+#pragma unroll
+          for (int v = 0; v < 4; ++v) hist[v] += (n >> (4 * v)) & 0x000F000Fu;
+        }
+      }
+    }
+    flow_report2(slot, cnt, rec, hist);
+  }
+  if (mine) {
+    const long long N = (long long)L * L;
+    uint32_t* dst = reinterpret_cast<uint32_t*>(A.state + (size_t)((step0 + n_steps) & 1) * N);
+#pragma unroll
+    for (int k = 0; k < V; ++k)
+      if ((uint32_t)k < h && dcheck((y0 + k) * Lh + p < L * Lh, err, kSiteTileWrite))
+        dst[(y0 + k) * Lh + p] = w[k];
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Layered schedule: the arms of a segment (at most two, no opposite pair) of
+// every cell, four cells of a row per group; the tag of a part in the top 16
+// bits of a cell's word, a step advancing it by 4.  ONE: one group per thread,
+// its words and the step's draws in registers; otherwise the draws are made
+// again for every segment.
+// ---------------------------------------------------------------------------
+template <int RNG_WORDS, bool CMP64, bool ONE, int NT>
+__global__ void __launch_bounds__(NT + 32, 1)
+    k_flow2_layer(const __grid_constant__ LatticeArgs A, const __grid_constant__ Flow2Geom G,
+                  WaveHdr* H, uint32_t* copy, long long n_steps, int every) {
+  __shared__ union {
+    Flow2Smem sweep;
+    VolumeArgs vol;
+  } U;
+  Ctrl* const ctl = A.ctrl;
+  unsigned int* const err = &ctl->error;
+  const long long step0 = *(volatile long long*)&ctl->sweep;
+  const uint32_t tag0 = *(volatile uint32_t*)copy + 4u;
+  if (blockIdx.x == 0) {
+    flow_books(A, U.vol, H, (int)gridDim.x - 1, copy,
+               tag0 + 4u * (uint32_t)((unsigned long long)n_steps & 0xFFFFFFu), step0, n_steps,
+               every);
+    return;
+  }
+  Flow2Smem& S = U.sweep;
+  uint32_t* const F = copy + kFlow2Head;
+  const uint32_t t_lo = (blockIdx.x - 1u) * G.per_block, t_hi = min(t_lo + G.per_block, G.items);
+  const int warps = (int)min((t_hi - t_lo + 31u) / 32u, (uint32_t)(NT / 32));
+  flow2_setup(S, A, NT + 32);
+  __syncthreads();
+  if (threadIdx.x >= NT) {
+    flow_clerk([&](long long s) { return (unsigned long long)layer_plan(s, A.keys); }, S.ring,
+               warps, H, err, step0, n_steps, every);
+    return;
+  }
+  if ((int)(threadIdx.x >> 5) >= warps) return;
+  const unsigned int full = 0xFFFFFFFFu;
+  const uint32_t L = (uint32_t)A.L, q = A.q;
+  const uint32_t Gx = G.groups_x, pitch = 4u * Gx;  // groups per row; the copy's row pitch
+  const long long N = (long long)L * L;
+  const uint32_t first = t_lo + (threadIdx.x & ~31u), lane = threadIdx.x & 31u;
+
+  // a group: its row, its x group and its number of cells (2 in a row's last
+  // group when L % 4 == 2)
+  struct Group {
+    uint32_t y, x, n;
+  };
+  auto locate = [&](uint32_t i) {
+    Group gr;
+    gr.y = fdiv(i, G.div_row);
+    gr.x = i - gr.y * Gx;
+    gr.n = min(4u, L - 4u * gr.x);
+    return gr;
+  };
+  uint32_t w[4] = {0u, 0u, 0u, 0u};  // the group's cells
+  CellWords<RNG_WORDS> draw[4];
+  {
+    const uint16_t* src = A.state + (size_t)(step0 & 1) * N;
+    for (uint32_t i0 = first; i0 < t_hi; i0 += NT) {
+      const uint32_t i = min(i0 + lane, t_hi - 1u);
+      const Group gr = locate(i);
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        w[c] = ((uint32_t)c < gr.n) ? __ldcg(src + (size_t)gr.y * L + 4u * gr.x + c) : 0u;
+      if (i0 + lane < t_hi)
+        st_flow4(F + (size_t)gr.y * pitch + 4u * gr.x,
+                 make_uint4(w[0] | (tag0 << 16), w[1] | (tag0 << 16), w[2] | (tag0 << 16),
+                            w[3] | (tag0 << 16)));
+    }
+  }
+  uint16_t* const dst = A.state + (size_t)((step0 + n_steps) & 1) * N;
+
+  for (long long rel = 0; rel < n_steps; ++rel) {
+    const long long step = step0 + rel;
+    FlowSlot& slot = S.ring[rel % kWaveRing];
+    const uint32_t tag = tag0 + 4u * (uint32_t)((unsigned long long)rel & 0xFFFFFFu);
+    const StepDraw sd = step_draw((uint32_t)((unsigned long long)step & 0xFFFFFFFFu),
+                                  (uint32_t)((unsigned long long)step >> 32), A.keys);
+    auto draw_group = [&](const Group& gr) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        draw[c] = cell_words<RNG_WORDS>(gr.y * L + 4u * gr.x + (uint32_t)c, sd, A.keys);
+    };
+    if (ONE) draw_group(locate(min(first + lane, t_hi - 1u)));
+    if (!flow_ready(slot, rel, H, err)) return;
+    const uint32_t plan = (uint32_t)slot.plan;
+    const Tables2& Tb = S.Tb[slot.g];
+    const bool rec = step_recorded(every, step);
+    const int nseg = 1 + __popc(plan >> 9);
+    TileCounts cnt{0, 0, 0};
+    uint32_t hist[4] = {0u, 0u, 0u, 0u};
+    for (int j = 0; j < nseg; ++j) {
+      const uint32_t arms = layer_segment(plan, j);
+      const int na = (int)(arms & 3u);
+      const bool last = j == nseg - 1;
+      const uint32_t need = (tag + (uint32_t)j) << 16;
+      const uint32_t out = (last ? tag + 4u : tag + 1u + (uint32_t)j) << 16;
+      for (uint32_t i0 = first; i0 < t_hi; i0 += NT) {
+        const bool mine = i0 + lane < t_hi;
+        const Group gr = locate(min(i0 + lane, t_hi - 1u));
+        uint32_t* const own = F + (size_t)gr.y * pitch + 4u * gr.x;
+        if (!ONE) {
+          const uint4 v = __ldcg(reinterpret_cast<const uint4*>(own));
+          w[0] = v.x & 0xFFFFu;
+          w[1] = v.y & 0xFFFFu;
+          w[2] = v.z & 0xFFFFu;
+          w[3] = v.w & 0xFFFFu;
+          draw_group(gr);
+        }
+        uint32_t nb[2][4];
+        for (unsigned int spins = 0;;) {
+          uint32_t late = 0u;
+#pragma unroll
+          for (int s = 0; s < 2; ++s) {
+            if (s >= na) continue;
+            const uint32_t a = (arms >> (2 + 2 * s)) & 3u;
+            if (a >= 2u) {
+              const uint32_t yn = (a == 2u) ? (gr.y + 1u == L ? 0u : gr.y + 1u)
+                                            : (gr.y == 0u ? L - 1u : gr.y - 1u);
+              const uint4 v = ld_flow4(F + (size_t)yn * pitch + 4u * gr.x);
+              nb[s][0] = v.x;
+              nb[s][1] = v.y;
+              nb[s][2] = v.z;
+              nb[s][3] = v.w;
+              late |= behind(v.x, need) | behind(v.y, need);
+              if (gr.n == 4u) late |= behind(v.z, need) | behind(v.w, need);
+            } else {
+              // the group's own cells serve but for the one at its end: arm a^1
+              // does not change in the segment
+              const uint32_t x = (a == 0u) ? (4u * gr.x + gr.n == L ? 0u : 4u * gr.x + 4u)
+                                           : (gr.x == 0u ? L - 1u : 4u * gr.x - 1u);
+              const uint32_t e = ld_flow(F + (size_t)gr.y * pitch + x);
+              late |= behind(e, need);
+              const bool plus = a == 0u;
+              nb[s][0] = plus ? w[1] : e;
+              nb[s][1] = plus ? (gr.n == 2u ? e : w[2]) : w[0];
+              nb[s][2] = plus ? w[3] : w[1];
+              nb[s][3] = plus ? e : w[2];
+            }
+          }
+          if (__all_sync(full, (int32_t)late >= 0)) break;
+          if ((++spins & 255u) == 0u && flow_stop(spins, H, err)) return;
+        }
+        if (mine) {
+          uint32_t pk = 0;
+#pragma unroll
+          for (int s = 0; s < 2; ++s) {
+            if (s >= na) continue;
+            const uint32_t a = (arms >> (2 + 2 * s)) & 3u;
+            auto pass = [&](auto arm_c) {
+              constexpr int ARM = decltype(arm_c)::value;
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                if ((uint32_t)c >= gr.n) continue;
+                uint32_t acc[4], kk[4];
+                split_draws<RNG_WORDS>(draw[c].u, draw[c].p, q, acc, kk);
+                const uint32_t n2 = twice(nb[s][c], false);
+                const uint32_t p2 = (ARM & 1) ? n2 << 4 : n2 >> 4;  // nibble a^1 to nibble a
+                w[c] = update_arm2<CMP64, ARM>(twice(w[c], false), p2, acc[ARM], kk[ARM], q, Tb,
+                                               pk) & 0xFFFFu;
+              }
+            };
+            if (a == 0u)
+              pass(std::integral_constant<int, 0>{});
+            else if (a == 1u)
+              pass(std::integral_constant<int, 1>{});
+            else if (a == 2u)
+              pass(std::integral_constant<int, 2>{});
+            else
+              pass(std::integral_constant<int, 3>{});
+          }
+          cnt.add(pk);
+          st_flow4(own, make_uint4(w[0] | out, w[1] | out, w[2] | out, w[3] | out));
+          if (last && rec) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const uint32_t n = ((uint32_t)c < gr.n) ? count_word4(w[c]) : 0u;
+#pragma unroll
+              for (int v = 0; v < 4; ++v) hist[v] += (n >> (4 * v)) & 0x000F000Fu;
+            }
+          }
+          if (last && rel == n_steps - 1) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              if ((uint32_t)c < gr.n &&
+                  dcheck((long long)gr.y * L + 4u * gr.x + c < N, err, kSiteLayer))
+                dst[(size_t)gr.y * L + 4u * gr.x + c] = (uint16_t)w[c];
+          }
+        }
+        __syncwarp();
+      }
+    }
+    flow_report2(slot, cnt, rec, hist);
+  }
+}
+
+template <int V, int NT>
+const void* flow2_kernel(int rng_words, bool cmp64) {
+  if (rng_words == 1)
+    return cmp64 ? (const void*)k_flow2<1, true, V, NT> : (const void*)k_flow2<1, false, V, NT>;
+  return cmp64 ? (const void*)k_flow2<2, true, V, NT> : (const void*)k_flow2<2, false, V, NT>;
+}
+
+template <bool ONE, int NT>
+const void* flow2_layer_kernel(int rng_words, bool cmp64) {
+  if (rng_words == 1)
+    return cmp64 ? (const void*)k_flow2_layer<1, true, ONE, NT>
+                 : (const void*)k_flow2_layer<1, false, ONE, NT>;
+  return cmp64 ? (const void*)k_flow2_layer<2, true, ONE, NT>
+               : (const void*)k_flow2_layer<2, false, ONE, NT>;
+}
+
+// Adopts the kernel of `form` for `items` spread over the SMs, one item per
+// thread (one) or any number, if they fit.
+struct Flow2Form {
+  int v, threads;
+  const void* (*kernel)(int rng_words, bool cmp64);
+};
+bool adopt(Flow2Plan* P, const Flow2Form& form, int rng_words, bool cmp64, long long items,
+           bool one) {
+  if (one && items > (long long)(sm_count() - 1) * form.threads) return false;
+  const void* const kernel = form.kernel(rng_words, cmp64);
+  const long long room =
+      std::min(sm_count(), flow_resident_blocks(kernel, form.threads + 32)) - 1;
+  if (room < 1 || (one && items > room * form.threads)) return false;
+  const long long share = ((items + room - 1) / room + 31) / 32 * 32;
+  P->kernel = kernel;
+  P->threads = form.threads + 32;
+  P->geom.items = (uint32_t)items;
+  P->geom.per_block = (uint32_t)share;
+  P->blocks = (int)((items + share - 1) / share);
+  return true;
+}
+
+// The strips of the checkerboard sweep, the first that fits: the fewest rows a
+// thread, then the fewest threads (the most registers) a block.  us per MC step
+// on GB300, with the sides where each ends (151 blocks): one row and 480
+// threads (380), 992 (547): 512^2 2.74 against 2.82 with two rows and 480; two
+// rows, 736 (667): 640^2 3.38 against 3.61 with 992; 992 (774): 768^2 4.49
+// against 5.08 with four and 736; four rows, 736 (943): 896^2 6.0 against 6.35;
+// 992 (1094): 1024^2 7.6 against 11.9 with eight rows and 480, which hides too
+// little latency.
+const Flow2Form kStrips[] = {{1, 480, flow2_kernel<1, 480>}, {1, 992, flow2_kernel<1, 992>},
+                             {2, 736, flow2_kernel<2, 736>}, {2, 992, flow2_kernel<2, 992>},
+                             {4, 736, flow2_kernel<4, 736>}, {4, 992, flow2_kernel<4, 992>}};
+// The layered sweep: one group a thread (512^2 4.3 us per step), or several with
+// as many warps as fit (1024^2 14.6 us with 992 threads, 16.4 with 736, 17.3
+// with 480; 4096^2 195, 201, 240).
+const Flow2Form kLayerOne = {0, 480, flow2_layer_kernel<true, 480>};
+const Flow2Form kLayerMany = {0, 992, flow2_layer_kernel<false, 992>};
+
+}  // namespace
+
+Flow2Plan flow2_plan(int L, int schedule, int rng_words, bool cmp64) {
+  Flow2Plan P{};
+  if (schedule == CVF_SCHED_LAYERED) {
+    const long long gx = (L + 3) / 4, groups = gx * L;
+    P.geom.groups_x = (uint32_t)gx;
+    P.geom.div_row = make_fastdiv((uint32_t)gx);
+    P.copy_words = (size_t)kFlow2Head + 4 * (size_t)groups;
+    if (!adopt(&P, kLayerOne, rng_words, cmp64, groups, true))
+      adopt(&P, kLayerMany, rng_words, cmp64, groups, false);
+    return P;
+  }
+  const long long Lh = L / 2;
+  P.geom.div_row = make_fastdiv((uint32_t)Lh);
+  P.copy_words = (size_t)kFlow2Head + (size_t)(Lh * L);
+  for (const Flow2Form& form : kStrips)
+    if (adopt(&P, form, rng_words, cmp64, Lh * ((L + form.v - 1) / form.v), true)) break;
+  return P;
+}
+
+cudaError_t launch_flow2(const LatticeArgs& A, const Flow2Plan& P, WaveHdr* H, long long n_steps,
+                         int every, cudaStream_t s) {
+  uint32_t* copy = reinterpret_cast<uint32_t*>(H + 1);
+  const cudaError_t e = cudaMemsetAsync(H, 0, sizeof(WaveHdr), s);
+  if (e != cudaSuccess) return e;
+  void* args[6] = {const_cast<LatticeArgs*>(&A), const_cast<Flow2Geom*>(&P.geom), &H, &copy,
+                   &n_steps, &every};
+  return cudaLaunchCooperativeKernel(P.kernel, dim3(P.blocks + 1), dim3(P.threads), args, 0, s);
+}
+
+}  // namespace cvf

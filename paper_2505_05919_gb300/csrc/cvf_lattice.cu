@@ -13,6 +13,7 @@
 
 #include "cvf.h"
 #include "cvf_device.cuh"
+#include "cvf_flow2.cuh"
 #include "cvf_host.h"
 #include "cvf_lattice.cuh"
 #include "cvf_tile.cuh"
@@ -408,41 +409,6 @@ __global__ void __launch_bounds__(kThreads, kSweepBlocksPerSM)
 // ---------------------------------------------------------------------------
 constexpr int kLayerLaunches = 3;
 
-// Plan word: bits 2i..2i+1 the arm of pass i, bit 8 + i set when pass i
-// opens a new launch (i = 1..3).
-__device__ uint32_t layer_plan(long long step, const RoundKeys& K) {
-  const Words4 r = philox(kCellLayers, (uint32_t)((unsigned long long)step & 0xFFFFFFFFu),
-                          (uint32_t)((unsigned long long)step >> 32), kTagLayers, K);
-  const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
-  int order[4] = {0, 1, 2, 3};
-  for (int i = 3; i >= 1; --i) {
-    const int j = (int)__umulhi(rw[3 - i], (uint32_t)(i + 1));
-    const int t = order[i];
-    order[i] = order[j];
-    order[j] = t;
-  }
-  uint32_t plan = 0, in_launch = 0;
-  for (int i = 0; i < 4; ++i) {
-    const int a = order[i];
-    if (in_launch & (1u << (a ^ 1))) {
-      plan |= 1u << (8 + i);
-      in_launch = 0;
-    }
-    in_launch |= 1u << a;
-    plan |= (uint32_t)a << (2 * i);
-  }
-  return plan;
-}
-
-__device__ int layer_plan_arms(uint32_t plan, int j, int* arms) {
-  int launch = 0, n = 0;
-  for (int i = 0; i < 4; ++i) {
-    if (i > 0 && ((plan >> (8 + i)) & 1u)) ++launch;
-    if (launch == j && n < 2) arms[n++] = (int)((plan >> (2 * i)) & 3u);
-  }
-  return n;
-}
-
 // The partner of arm a of the cell in half `hi` of word `own` (at column p
 // of row y), moved to bits 16..18: arm a^1 of the neighbour in direction a.
 __device__ __forceinline__ uint32_t layer_partner(int a, int hi, uint32_t own, const uint32_t* buf,
@@ -484,11 +450,11 @@ __global__ void __launch_bounds__(kThreads) k_layer(LatticeArgs A, int launch) {
     } else {
       plan = (uint32_t)ctl->plan;
     }
-    int arms[2] = {0, 0};
-    const int n = layer_plan_arms(plan, launch, arms);
+    const uint32_t segment = layer_segment(plan, launch);
+    const int n = (int)(segment & 3u);
     s_n = n;
-    s_arm[0] = arms[0];
-    s_arm[1] = arms[1];
+    s_arm[0] = (int)((segment >> 2) & 3u);
+    s_arm[1] = (int)((segment >> 4) & 3u);
     const int nlaunch = 1 + __popc(plan >> 9);
     s_rec = (n > 0 && launch == nlaunch - 1 && step_recorded(ctl->record_every, ctl->sweep)) ? 1 : 0;
   }
@@ -683,6 +649,9 @@ struct cvf_handle {
   int graph_steps;
   WaveHdr* wave;  // scratch of the wavefront sweep (allocated when first chosen)
   size_t wave_bytes;
+  Flow2Plan flow;     // the dataflow sweep (no blocks: the lattice is too large for it)
+  WaveHdr* flow_hdr;  // its scratch and, behind it, its tagged copy
+  bool use_flow;      // the automatic choice takes it
 };
 
 namespace {
@@ -700,6 +669,7 @@ void release(cvf_handle* h) {
   if (!h) return;
   if (h->graph) cudaGraphExecDestroy(h->graph);
   if (h->wave) cudaFree(h->wave);
+  if (h->flow_hdr) cudaFree(h->flow_hdr);
   if (h->own_state && h->state) cudaFree(h->state);
   if (h->ctrl) cudaFree(h->ctrl);
   if (h->ring) cudaFree(h->ring);
@@ -911,7 +881,10 @@ int wave_scratch(cvf_handle* h, int shape) {
   return CVF_OK;
 }
 
-// The automatic configuration: the resident form for small lattices; the
+// The automatic configuration of the lattices that the dataflow sweep does not
+// take (Flow2Plan; it is faster wherever it fits: 64^2 1.8 against 2.7 us per
+// step with the resident form, 258^2 1.9 / 7.9 tiled, 512^2 2.7 / 7.0 and 1024^2
+// 7.6 / 11.2 with the wavefront): the resident form for small lattices; the
 // wavefront sweep from 256^2 up, with the tiled sweep's shape rule (the
 // largest shape with at least as many tiles as the tiled sweep has resident
 // blocks: the fastest wavefront shape at 768^2, 1536^2, 2048^2 and from
@@ -926,6 +899,11 @@ int wave_scratch(cvf_handle* h, int shape) {
 // filled last round of tiles costs less the more tiles a step has, but the
 // wavefront stays ahead).
 constexpr int kWaveAutoMin = 256;
+// The layered schedule runs as a dataflow sweep (cvf_flow2.cu) up to this side:
+// it is faster than a launch per segment at every side measured (1024^2 14.6
+// against 31.8 us per step, 2048^2 55.5 / 80.2, 4096^2 195 / 260), but its copy
+// doubles the lattice's memory (4 bytes a cell).
+constexpr int kFlowLayerMaxSide = 16384;
 int auto_config(const cvf_handle* h) {
   const cvf_params& p = h->p;
   if (p.schedule == CVF_SCHED_CHECKERBOARD && p.L <= kResAutoSide &&
@@ -978,6 +956,8 @@ int recount_into_ctrl(cvf_handle* h) {
 int build_graph(cvf_handle* h) {
   if (h->graph) return CVF_OK;
   cudaGraph_t g = nullptr;
+  if (!h->cap_stream)
+    CVF_CUDA_CHECK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   CVF_CUDA_CHECK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t le = cudaSuccess;
   for (int i = 0; i < kGraphSteps && le == cudaSuccess; ++i) le = enqueue_step(h, h->cap_stream);
@@ -1031,7 +1011,6 @@ int cvf_create(const cvf_params* p, void* stream, void* dev_state, cvf_handle** 
       return code_;                                                               \
     }                                                                             \
   } while (0)
-  CREATE_CHECK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   if (dev_state) {
     h->state = reinterpret_cast<uint16_t*>(dev_state);
     h->own_state = false;
@@ -1065,9 +1044,22 @@ int cvf_create(const cvf_params* p, void* stream, void* dev_state, cvf_handle** 
   h->args.keys = make_round_keys(p->seed);
   h->args.L = p->L;
   h->args.q = (uint32_t)p->q;
+  if (p->schedule == CVF_SCHED_CHECKERBOARD || p->L <= kFlowLayerMaxSide)
+    h->flow = flow2_plan(p->L, p->schedule, p->rng_words, h->cmp64);
+  if (h->flow.blocks > 0) {
+    const size_t bytes = sizeof(WaveHdr) + sizeof(uint32_t) * h->flow.copy_words;
+    if (cudaMalloc(reinterpret_cast<void**>(&h->flow_hdr), bytes) != cudaSuccess) {
+      cudaGetLastError();  // no room for the copy: the lattice runs without it
+      h->flow_hdr = nullptr;
+      h->flow.blocks = 0;
+    } else {
+      CREATE_CHECK(cudaMemsetAsync(h->flow_hdr, 0, bytes, h->stream));
+      h->use_flow = true;
+    }
+  }
   {
     const int cfg = auto_config(h);
-    if (is_wave(cfg)) {
+    if (is_wave(cfg) && !h->use_flow) {
       rc = wave_scratch(h, cfg - kWave);
       if (rc) {
         release(h);
@@ -1104,6 +1096,15 @@ int cvf_sweep(cvf_handle* h, int64_t n_sweeps, int32_t record_every) {
     return set_error(CVF_EINVAL, "n_sweeps=%lld, record_every=%d must be >= 0",
                      (long long)n_sweeps, record_every);
   if (n_sweeps == 0) return CVF_OK;
+  if (h->use_flow) {
+    constexpr long long kChunk = 1ll << 30;  // the launch's step counters are 32-bit
+    for (long long done = 0; done < n_sweeps; done += kChunk)
+      CVF_CUDA_CHECK(launch_flow2(h->args, h->flow, h->flow_hdr,
+                                  std::min<long long>(kChunk, n_sweeps - done), record_every,
+                                  h->stream));
+    h->sweep_host += n_sweeps;
+    return CVF_OK;
+  }
   k_set_record<<<1, 32, 0, h->stream>>>(h->ctrl, record_every);
   if (is_wave(h->tile)) {
     // one persistent launch per 2^30 steps (the launch's step counters are 32-bit)
@@ -1285,6 +1286,8 @@ int cvf_set_tiles(cvf_handle* h, int32_t config) {
     const int rc = wave_scratch(h, config - kWave);
     if (rc) return rc;
   }
+  // the layered schedule has no tiles to choose
+  h->use_flow = h->flow.blocks > 0 && (config < 0 || h->p.schedule == CVF_SCHED_LAYERED);
   if (config < 0) config = auto_config(h);
   set_tile(h, config);
   return CVF_OK;

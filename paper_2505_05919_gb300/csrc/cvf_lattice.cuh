@@ -93,6 +93,8 @@ struct WaveHdr {
   WaveMove vring[kWaveRing];
   WaveAcc acc[kWaveRing];
 };
+// (the dataflow sweeps' copy, read as 16-byte vectors, lies behind it)
+static_assert(sizeof(WaveHdr) % 128 == 0, "WaveHdr ends on a 128-byte boundary");
 // Co-resident blocks of the wavefront kernel for a tile shape (0 if none).
 int wave_blocks(int rng_words, bool cmp64, int shape);
 // Clears the scratch (scratch_bytes) and launches the call's steps.

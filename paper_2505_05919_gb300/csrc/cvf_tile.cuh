@@ -110,7 +110,7 @@ __device__ __forceinline__ uint32_t update_arm2(uint32_t w2, uint32_t p2, uint32
   const uint32_t e = k * (4u * q) + s4;
   const uint32_t vR = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(Tb.prop) + e);
   const uint32_t nR = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(Tb.next) + e);
-  constexpr uint32_t mask = 0x000F000Fu << (4 * ARM);
+  constexpr uint32_t mask = 0x00070007u << (4 * ARM);  // bit 3 of p2's nibbles may be anything
   const uint32_t x = (w2 & ~mask) | (p2 & mask);
   const uint32_t f = ((x ^ vR) + 0x11117777u) & 0x88888888u;
   const uint32_t copy = (threadIdx.x & 1u) * (uint32_t)(4 * kRowCopy);
@@ -181,19 +181,17 @@ __device__ __forceinline__ void draws(uint32_t c, uint32_t, uint32_t, const Keys
 }
 
 // Update the cell in half `hi` of word `own` (its four arms in order, each
-// seeing the earlier ones); xm / xp are the words to the left / right, ym /
-// yp the words of the rows y-1 / y+1.  Accepted moves add their packed count
-// changes to pk; with s_hist4 (recorded steps) the cell's N_q' is counted.
-// HI = 0 / 1 fixes the half at compile time (a warp whose lanes all update
-// the same half); HI = -1 takes it from hi_rt.
-template <int RNG_WORDS, bool CMP64, int HI = -1, typename KEYS>
-__device__ __forceinline__ uint32_t update_in_word(uint32_t own, uint32_t xm_word,
-                                                   uint32_t xp_word, uint32_t ym_word,
-                                                   uint32_t yp_word, int hi_rt, uint32_t c,
-                                                   uint32_t s_lo, uint32_t s_hi,
-                                                   const KEYS& keys, uint32_t q,
-                                                   const Tables2& Tb, uint32_t& pk,
-                                                   uint32_t* s_hist4) {
+// seeing the earlier ones) with its draws; xm / xp are the words to the left /
+// right (only the one on the cell's side is read), ym / yp the words of the
+// rows y-1 / y+1; bit 3 of a neighbour's nibbles may be anything.  Accepted
+// moves add their packed count changes to pk; the result is the cell in both
+// halves.  HI = 0 / 1 fixes the half at compile time (a warp whose lanes all
+// update the same half); HI = -1 takes it from hi_rt.
+template <bool CMP64, int HI = -1>
+__device__ __forceinline__ uint32_t update_cell(uint32_t own, uint32_t xm_word, uint32_t xp_word,
+                                                uint32_t ym_word, uint32_t yp_word, int hi_rt,
+                                                const uint32_t acc[4], const uint32_t kk[4],
+                                                uint32_t q, const Tables2& Tb, uint32_t& pk) {
   // partners: arm 0 (+x) <-> arm 1 of the +x cell, arm 1 (-x) <-> arm 0 of
   // the -x cell, arm 2 (+y) <-> arm 3 of the +y cell, arm 3 (-y) <-> arm 2 of
   // the -y cell.  Each lies in the byte it has to go to or a whole byte
@@ -208,14 +206,34 @@ __device__ __forceinline__ uint32_t update_in_word(uint32_t own, uint32_t xm_wor
   const uint32_t B = __byte_perm(hi ? own : xm_word, ym_word, sel);
   const uint32_t p2 = ((A >> 4) & 0x0F0F0F0Fu) | ((B << 4) & 0xF0F0F0F0u);
   uint32_t w = twice(own, hi);
-  uint32_t acc[4], kk[4];
-  draws<RNG_WORDS>(c, s_lo, s_hi, keys, q, acc, kk);
   w = update_arm2<CMP64, 0>(w, p2, acc[0], kk[0], q, Tb, pk);
   w = update_arm2<CMP64, 1>(w, p2, acc[1], kk[1], q, Tb, pk);
   w = update_arm2<CMP64, 2>(w, p2, acc[2], kk[2], q, Tb, pk);
   w = update_arm2<CMP64, 3>(w, p2, acc[3], kk[3], q, Tb, pk);
-  if (s_hist4) hist_add_cell(s_hist4, count_word4(w));
+  return w;
+}
+
+// Word `own` with the cell of half `hi` replaced by the one in w's halves.
+__device__ __forceinline__ uint32_t put_cell(uint32_t own, uint32_t w, bool hi) {
   return __byte_perm(own, w, hi ? 0x5410u : 0x3254u);
+}
+
+// The same with the cell's draws made here; with s_hist4 (recorded steps) the
+// cell's N_q' is counted.  Returns the updated word.
+template <int RNG_WORDS, bool CMP64, int HI = -1, typename KEYS>
+__device__ __forceinline__ uint32_t update_in_word(uint32_t own, uint32_t xm_word,
+                                                   uint32_t xp_word, uint32_t ym_word,
+                                                   uint32_t yp_word, int hi_rt, uint32_t c,
+                                                   uint32_t s_lo, uint32_t s_hi,
+                                                   const KEYS& keys, uint32_t q,
+                                                   const Tables2& Tb, uint32_t& pk,
+                                                   uint32_t* s_hist4) {
+  uint32_t acc[4], kk[4];
+  draws<RNG_WORDS>(c, s_lo, s_hi, keys, q, acc, kk);
+  const uint32_t w = update_cell<CMP64, HI>(own, xm_word, xp_word, ym_word, yp_word, hi_rt, acc,
+                                            kk, q, Tb, pk);
+  if (s_hist4) hist_add_cell(s_hist4, count_word4(w));
+  return put_cell(own, w, ((HI >= 0) ? HI : hi_rt) != 0);
 }
 
 // Staged input: rows y0-2 .. y0+TR+1 and words p0-4 .. p0+TW+3 (a 16-byte

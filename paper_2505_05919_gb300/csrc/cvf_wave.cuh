@@ -109,63 +109,198 @@ __device__ inline void wave_commit(Ctrl* ctl, const VolumeArgs& vol, cvf_obs* ri
   st_release_u32(&H->committed, (unsigned int)(r + 1));
 }
 
+// ---------------------------------------------------------------------------
 // The volume engine (Sec. II.B step 1), run by the first two warps of one
 // block: the move of every step of a call of n_steps, and of the first step of
-// the next one, each from the move before it and published in the ring while
-// at most kWaveRing steps are ahead of the commits.  A proposal that would
-// change the gate waits for the commit of the step before and is decided with
-// its bonds.  sV is a shared copy of the parameters.
+// the next one, published in the ring while at most kWaveRing steps are ahead
+// of the commits.  While no proposal would change the gate, a move follows from
+// the volume after the move before it and the step's draws alone, so a pass
+// decides kEngDepth steps at once over the tree of outcomes: node i (heap
+// order, lane i) is the move of step t0 + depth(i) from the state that the
+// accept / reject outcomes on its path lead to.  An FP64 instruction occupies
+// the pipe for a whole warp whatever the number of active lanes, so a pass
+// costs about what one decision costs (step by step 64^2 would take the 2 to 4
+// us of a decision per step).  Each node runs the IEEE operations of
+// volume_decide_pair in the same order, so every move equals the step-by-step
+// chain's.  A proposal that would change the gate ends the walk; it waits for
+// the commit of the step before and is decided with its bonds.  sV is a shared
+// copy of the parameters.
+// ---------------------------------------------------------------------------
+constexpr int kWaveTree = 5;  // steps per pass: 31 nodes
+
+struct WaveTree {
+  double log_ratio[32];  // N log(V'/V) of the nodes, from warp 1
+  double exchange;       // volume_decide_pair's
+  double V, u;           // the state after the last move decided
+  int g, acc;
+  int flip;              // the next move would change the gate
+  int settled;           // steps the pass decided
+  int go;
+};
+
+// The number of shells inside the cutoff at v, from a guess: the test holds for
+// a prefix of the ascending shells, so a guess is moved to the prefix's end.
+__device__ __forceinline__ int lj_shells_near(const VolumeArgs& V, double v, int k) {
+  const bool cubic = V.dim == 3;
+  auto inside = [&](int i) {
+    const double key = cubic ? (V.shell_d2[i] * v) * v : V.shell_d2[i] * v;
+    return key < V.cutoff2;
+  };
+  while (k < V.nshell && inside(k)) ++k;
+  while (k > 0 && !inside(k - 1)) --k;
+  return k;
+}
+
 __device__ inline void wave_engine(Ctrl* ctl, const VolumeArgs& sV, const RoundKeys& keys,
                                    WaveHdr* H, long long step0, long long n_steps) {
-  __shared__ double s_xch;
-  __shared__ VolumeResult s_res;
-  __shared__ int s_go;
+  __shared__ WaveTree T;
+  const unsigned int full = 0xFFFFFFFFu;
   unsigned int* const err = &ctl->error;
-  const int role = (int)(threadIdx.x >> 5);
+  const int role = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31u);
+  const int n1 = lane + 1;       // 1-based heap index: children 2 n1 (reject), 2 n1 + 1 (accept)
+  const int d = 31 - __clz(n1);  // depth (lane 31: below the tree, not used)
+  const double Nd = (double)sV.N;
   volatile Ctrl* c = ctl;
-  VolumeResult cur;
-  cur.V = c->next_V;
-  cur.u = c->next_u;
-  cur.g = c->next_g;
-  cur.accepted = c->next_acc;
-  if (threadIdx.x == 0) wave_publish(H, 0, cur);
-  bool alive = true;
-  for (long long r = 1; r <= n_steps; ++r) {
-    if (threadIdx.x == 0)
-      s_go = (r < kWaveRing) ? 1
-                             : (wave_wait_geq(&H->committed, (unsigned int)(r - kWaveRing + 1), H,
-                                              err) ? 1 : 0);
-    engine_sync();
-    if (!s_go) {
-      alive = false;
-      break;
-    }
-    VolumeResult res;
-    const bool ok = volume_decide_pair<3>(role, sV, step0 + r, cur.V, cur.u, cur.g, -1,
-                                          keys, &res, &s_xch);
-    if (!ok) {
-      // the proposal changes the gate: decide it with the bonds after step r - 1
-      if (threadIdx.x == 0) s_go = wave_wait_geq(&H->committed, (unsigned int)r, H, err) ? 1 : 0;
-      engine_sync();
-      if (!s_go) {
-        alive = false;
-        break;
-      }
-      const long long nhb = c->n_hb_raw;
-      volume_decide_pair<3>(role, sV, step0 + r, cur.V, cur.u, cur.g, nhb, keys, &res,
-                            &s_xch);
-    }
-    if (threadIdx.x == 0) s_res = res;  // valid in role 0's lanes
-    engine_sync();
-    cur = s_res;
-    engine_sync();  // every thread has read s_res before the next write
-    if (r < n_steps && threadIdx.x == 0) wave_publish(H, r, cur);
+  if (threadIdx.x == 0) {
+    VolumeResult cur;
+    cur.V = T.V = c->next_V;
+    cur.u = T.u = c->next_u;
+    cur.g = T.g = c->next_g;
+    cur.accepted = T.acc = c->next_acc;
+    T.flip = 0;
+    wave_publish(H, 0, cur);
   }
-  if (alive && threadIdx.x == 0) {
-    c->next_V = cur.V;
-    c->next_u = cur.u;
-    c->next_g = cur.g;
-    c->next_acc = cur.accepted;
+  engine_sync();
+  // one thread: the ring has room for the move of relative step r
+  auto room = [&](long long r) {
+    return r < kWaveRing ||
+           wave_wait_geq(&H->committed, (unsigned int)(r - kWaveRing + 1), H, err);
+  };
+  auto publish = [&](long long r) {  // T holds the move of relative step r
+    if (r >= n_steps) return true;   // the next call's first: stays in T
+    if (!room(r)) return false;
+    VolumeResult m;
+    m.V = T.V;
+    m.u = T.u;
+    m.g = T.g;
+    m.accepted = T.acc;
+    wave_publish(H, r, m);
+    return true;
+  };
+  int shells = 0;  // of the last pass's root, the guess of the next
+  for (long long r = 1; r <= n_steps;) {
+    const double bV = T.V, bu = T.u;
+    const int bg = T.g;
+    const long long t0 = step0 + r;
+    if (T.flip || !sV.volume_moves) {
+      // the gate would change: decide the move with the bonds after step r - 1
+      // (without volume moves every decision keeps the state)
+      if (threadIdx.x == 0)
+        T.go = (!T.flip || wave_wait_geq(&H->committed, (unsigned int)r, H, err)) ? 1 : 0;
+      engine_sync();
+      if (!T.go) return;
+      VolumeResult res;
+      volume_decide_pair<3>(role, sV, t0, bV, bu, bg, T.flip ? c->n_hb_raw : 0, keys, &res,
+                            &T.exchange);
+      engine_sync();  // both warps have read T
+      if (threadIdx.x == 0) {  // res is valid in role 0's lanes
+        T.V = res.V;
+        T.u = res.u;
+        T.g = res.g;
+        T.acc = res.accepted;
+        T.flip = 0;
+        T.go = publish(r) ? 1 : 0;
+      }
+      engine_sync();
+      if (!T.go) return;
+      ++r;
+      continue;
+    }
+    const long long st = t0 + d;
+    const Words4 w = philox(kCellVolume, (uint32_t)((unsigned long long)st & 0xFFFFFFFFu),
+                            (uint32_t)((unsigned long long)st >> 32), kTagVolume, keys);
+    const double u1 = u53(w.x, w.y), u2 = u53(w.z, w.w);
+    const double dV = (2.0 * u1 - 1.0) * sV.dV_max;
+    // the volume before the node's move: the accepted moves on its path, added
+    // in step order (lane 2^j - 1 holds the draw of depth j)
+    double Vo = bV;
+#pragma unroll
+    for (int j = 0; j < kWaveTree; ++j) {
+      const double dVj = __shfl_sync(full, dV, (1 << j) - 1);
+      if (j < d && ((n1 >> (d - 1 - j)) & 1)) Vo = Vo + dVj;
+    }
+    const double Vn = Vo + dV;
+    if (role == 1) {
+      T.log_ratio[lane] = Nd * log(Vn / Vo);
+      engine_sync();  // the logs are there
+      engine_sync();  // the pass is settled
+    } else {
+      const double vn = Vn / Nd;
+      const bool hard = vn < 1.0;
+      const int g_new = (vn < 2.0) ? 1 : 0;
+      const int k = lj_shells_near(sV, vn, shells);
+      shells = __shfl_sync(full, k, 0);
+      const double un = lj_energy_at(sV, vn, k);
+      // the energy before the move: that of the last accepted move on the path
+      // (its lane), else the root's
+      int src = -1;
+#pragma unroll
+      for (int j = 0; j < kWaveTree; ++j)
+        if (j < d && ((n1 >> (d - 1 - j)) & 1)) src = (n1 >> (d - j)) - 1;
+      const double uo_lane = __shfl_sync(full, un, src < 0 ? lane : src);
+      const double uo = (src < 0) ? bu : uo_lane;
+      const double J_eff = sV.J - sV.P * sV.v_HB;
+      const double du = un - uo;
+      const double t1 = Nd * du;
+      const double t2 = sV.P * dV;
+      const double t3 = ((double)(g_new - bg) * J_eff) * (double)0;
+      const double dH = (t1 + t2) - t3;
+      const double q = -dH / sV.kT;
+      engine_sync();  // the logs are there
+      const double arg = q + T.log_ratio[lane];
+      const bool met = u2 < exp(arg);
+      // walk the tree along the outcomes; every lane takes the same path
+      const bool node = lane < 31;
+      const bool flip = !hard && g_new != bg;
+      const unsigned int A = __ballot_sync(full, node && !hard && !flip && met);
+      const unsigned int U = __ballot_sync(full, node && flip);
+      double Vc = bV, uc = bu;
+      int nn = 1, j = 0;
+      bool go = true;
+      for (; j < kWaveTree && go && r + j <= n_steps; ++j) {
+        const int i = nn - 1;
+        if ((U >> i) & 1u) break;
+        const int a = (int)((A >> i) & 1u);
+        const double Vi = __shfl_sync(full, Vn, i), ui = __shfl_sync(full, un, i);
+        if (a) {
+          Vc = Vi;
+          uc = ui;
+        }
+        if (lane == 0) {
+          T.V = Vc;
+          T.u = uc;
+          T.acc = a;
+          go = publish(r + j);
+        }
+        go = __shfl_sync(full, go ? 1 : 0, 0) != 0;
+        nn = 2 * nn + a;
+      }
+      if (lane == 0) {
+        T.flip = (j < kWaveTree && r + j <= n_steps && ((U >> (nn - 1)) & 1u)) ? 1 : 0;
+        T.settled = j;
+        T.go = go ? 1 : 0;
+      }
+      engine_sync();  // the pass is settled
+    }
+    if (!T.go) return;
+    r += T.settled;
+  }
+  engine_sync();
+  if (threadIdx.x == 0) {
+    c->next_V = T.V;
+    c->next_u = T.u;
+    c->next_g = T.g;
+    c->next_acc = T.acc;
     c->ahead_state = 0;
   }
 }

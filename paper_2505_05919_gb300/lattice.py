@@ -81,11 +81,12 @@ class Lattice:
         """Tile shape of the sweep (0: 64x64, 1: 32x32, 2: 16x32 words; 3: the
         whole lattice resident in one thread-block cluster; 4, 5, 6: the
         shapes of 0, 1, 2 in the wavefront sweep, one persistent launch per
-        call; -1: automatic)."""
+        call; -1: automatic -- up to about L = 1094 a sweep without tiles)."""
         _capi.cvf_set_tiles(self.h, config)
 
     def tiles(self):
-        """(config, rows, words) of the sweep's tile shape."""
+        """(config, rows, words) of the sweep's tile shape (under the automatic
+        choice the rule's, also where the lattice runs without tiles)."""
         return _capi.cvf_get_tiles(self.h)
 
     def close(self) -> None:

@@ -609,3 +609,59 @@ def test_maximum_size_sampled_windows(L):
             want = lazy[y0 + margin:y0 + margin + inner, x0 + margin:x0 + margin + inner]
             got = lat.window(x0 + margin, y0 + margin, inner, inner)
             assert np.array_equal(got, want), (x0, y0)
+
+
+# The dataflow sweep at its edges: one and many blocks, blocks whose last warp is
+# partly empty, each strip height and block size at the sides where it begins or
+# ends (152 SMs), a last strip of two rows (L % 4 == 2), two-word draws, every q,
+# the 64-bit compare, gate flips, every step recorded; and the layered schedule's
+# groups (rows that end in half a group, one group a thread and several).
+DATAFLOW = [
+    (2, 80, 1, 0, {}),
+    (10, 60, 1, 0, dict(q=2, rng_words=2)),
+    (34, 30, 1, 0, dict(q=8)),
+    (66, 20, 7, 0, dict(init=oracle.INIT_ORDERED, rng_words=2)),
+    (380, 6, 2, 0, {}),
+    (382, 6, 1, 0, dict(rng_words=2)),
+    (546, 4, 1, 0, dict(kT=1e-3)),
+    (548, 4, 1, 0, dict(q=3)),
+    (670, 3, 1, 0, dict(rng_words=2)),
+    (776, 3, 0, 0, {}),
+    (778, 3, 1, 0, dict(q=5, rng_words=2)),
+    (946, 3, 1, 0, {}),
+    (1094, 3, 3, 0, dict(kT=1e-3)),
+    (6, 400, 1, 0, dict(gates=True)),
+    (70, 200, 1, 0, dict(gates=True)),
+    (2, 80, 1, 1, {}),
+    (34, 30, 1, 1, dict(rng_words=2)),
+    (66, 20, 3, 1, dict(kT=1e-3)),
+    (538, 4, 1, 1, dict(q=8)),
+    (542, 4, 1, 1, dict(rng_words=2)),
+    (6, 300, 1, 1, dict(gates=True)),
+]
+
+
+@pytest.mark.parametrize("L,K,every,layered,extra", DATAFLOW,
+                         ids=["L%d-%d" % (c[0], i) for i, c in enumerate(DATAFLOW)])
+def test_dataflow_sweep(L, K, every, layered, extra):
+    extra = dict(extra, schedule=oracle.SCHED_LAYERED if layered else 0)
+    if extra.pop("gates", False):
+        op = oracle.OracleParams(L=L, seed=40 + L, kT=1.0, P=0.5, J=0.0, v_HB=0.0, epsilon=0.0,
+                                 v_iso_init=1.98, dv_max_frac=0.02, **extra)
+    elif "kT" in extra:
+        op = oracle.OracleParams(L=L, seed=40 + L, **extra)
+    else:
+        op = oracle.physical_params(300.0, 0.1, L=L, seed=40 + L, dv_max_frac=0.02, **extra)
+    ref = oracle.Oracle(op)
+    want = ref.run(K, every)
+    with Lattice(params_from_dict(asdict(op))) as lat:
+        lat.sweep(K // 3, every)
+        lat.sweep(K - K // 3, every)
+        got, overflow = lat.drain()
+        s, o, counts = lat.state(), lat.observables(), lat.recount()
+    assert not overflow and len(got) == len(want)
+    assert np.array_equal(s, ref.state())
+    assert_obs_equal(o, ref.observables())
+    assert counts == (o["n_hb_raw"], o["n_coop"])
+    for i, (a, b) in enumerate(zip(got, want)):
+        assert_obs_equal(a, b, ("record", i))
