@@ -37,6 +37,7 @@
 #include "cvf_fastdiv.cuh"
 #include "cvf_host.h"
 #include "cvf_lattice.cuh"
+#include "cvf_observe.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -314,18 +315,12 @@ __global__ void __launch_bounds__(kThreads3) k_init3(uint32_t* __restrict__ stat
 
 // Full count of a lattice: N_HB_raw (arms 0, 2, 4 against arms 1, 3, 5 of
 // the +x, +y, +z neighbours, on edges with eta = 1) and N_sigma (equal pairs
-// among the six arms)
-// added to acc2[0], acc2[1]; N_q' added to hist[0..8).  Either may be NULL.
+// among the six arms) added to acc2[0], acc2[1].
 __global__ void __launch_bounds__(kThreads3) k_count3(const uint32_t* __restrict__ state,
                                                        uint32_t L, uint32_t L2, uint32_t N,
                                                        FastDiv div_L, FastDiv div_L2,
-                                                       unsigned long long* acc2,
-                                                       unsigned long long* hist) {
-  __shared__ unsigned long long s_cnt[8];
-  if (threadIdx.x < 8) s_cnt[threadIdx.x] = 0;
-  __syncthreads();
+                                                       unsigned long long* acc2) {
   uint32_t hb = 0, pairs = 0, unused = 0;
-  uint32_t h[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (uint32_t c = blockIdx.x * kThreads3 + threadIdx.x; c < N; c += gridDim.x * kThreads3) {
     const uint32_t z = fdiv(c, div_L2);
     const uint32_t rem = c - z * L2;
@@ -344,19 +339,13 @@ __global__ void __launch_bounds__(kThreads3) k_count3(const uint32_t* __restrict
     for (int v = 0; v < 8; ++v) {
       const uint32_t m = (cnt >> (4 * v)) & 15u;
       pairs += m * (m - 1u) / 2u;
-      h[v] += m;
     }
   }
-  if (hist)
-    for (int v = 0; v < 8; ++v)
-      if (h[v]) atomicAdd(&s_cnt[v], (unsigned long long)h[v]);
   block_sum3<kThreads3>(hb, pairs, unused);
-  if (threadIdx.x == 0 && acc2) {
+  if (threadIdx.x == 0) {
     atomicAdd(&acc2[0], (unsigned long long)hb);
     atomicAdd(&acc2[1], (unsigned long long)pairs);
   }
-  __syncthreads();
-  if (hist && threadIdx.x < 8 && s_cnt[threadIdx.x]) atomicAdd(&hist[threadIdx.x], s_cnt[threadIdx.x]);
 }
 
 // Step 2 of the MC step: one Metropolis move of every cube's configuration
@@ -757,16 +746,6 @@ __global__ void __launch_bounds__(kRes3Block) k_resident3(Args3 A, long long n_s
   for (uint32_t i = threadIdx.x; i < R * L2; i += blockDim.x) st[z0 * L2 + i] = cube[i];
 }
 
-// Observables of the committed state with N_q' from a count of the lattice.
-__global__ void k_observables3(const VolumeArgs* __restrict__ V, const Ctrl* ctl,
-                               const unsigned long long* hist, cvf_obs* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    cvf_obs o = make_obs(*V, ctl);
-    for (int v = 0; v < 8; ++v) o.n_state[v] = (long long)hist[v];
-    *out = o;
-  }
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -976,10 +955,9 @@ struct cvf3_handle {
   cvf_obs* ring;
   long long ring_cap;
   long long ring_tail;
-  cvf_obs* obs_dev;
   unsigned long long* table_dev;
   VolumeArgs* vol_dev;
-  unsigned long long* rc_dev;  // 10 counters: N_q'[8], N_HB_raw, N_sigma
+  unsigned long long* rc_dev;  // ten words of scratch, then ten of k_observe
   uint8_t* eta;                // cube configurations (eta moves only)
   unsigned long long* eta_table_dev;
   void* host_pinned;
@@ -1007,7 +985,6 @@ void release3(cvf3_handle* h) {
   if (h->own_state && h->state) cudaFree(h->state);
   if (h->ctrl) cudaFree(h->ctrl);
   if (h->ring) cudaFree(h->ring);
-  if (h->obs_dev) cudaFree(h->obs_dev);
   if (h->table_dev) cudaFree(h->table_dev);
   if (h->vol_dev) cudaFree(h->vol_dev);
   if (h->rc_dev) cudaFree(h->rc_dev);
@@ -1067,7 +1044,7 @@ int recount_into_ctrl3(cvf3_handle* h) {
   k_eta_bits3<<<h->grid_count, kThreads3, 0, h->stream>>>(h->args);
   k_count3<<<h->grid_count, kThreads3, 0, h->stream>>>(h->state, h->args.L, h->args.L2,
                                                         h->args.N, h->args.div_L, h->args.div_L2,
-                                                        &h->ctrl->acc_hb, nullptr);
+                                                        &h->ctrl->acc_hb);
   k_commit_counts<<<1, 32, 0, h->stream>>>(h->ctrl);
   k_volume_prologue<<<1, 32, 0, h->stream>>>(h->vol_dev, h->ctrl, h->args.keys);
   CVF_CUDA_CHECK(cudaGetLastError());
@@ -1137,10 +1114,9 @@ int cvf3_create(const cvf_params* p, void* stream, void* dev_state, cvf3_handle*
   }
   CREATE_CHECK(cudaMalloc(&h->ctrl, sizeof(Ctrl)));
   CREATE_CHECK(cudaMalloc(&h->ring, sizeof(cvf_obs) * (size_t)h->ring_cap));
-  CREATE_CHECK(cudaMalloc(&h->obs_dev, sizeof(cvf_obs)));
   CREATE_CHECK(cudaMalloc(&h->table_dev, sizeof(unsigned long long) * 66));
   CREATE_CHECK(cudaMalloc(&h->vol_dev, sizeof(VolumeArgs)));
-  CREATE_CHECK(cudaMalloc(&h->rc_dev, sizeof(unsigned long long) * 10));
+  CREATE_CHECK(cudaMalloc(&h->rc_dev, sizeof(unsigned long long) * 20));
   CREATE_CHECK(cudaMallocHost(&h->host_pinned, 4096));
   if (p->eta_moves) {
     CREATE_CHECK(cudaMalloc(&h->eta, (size_t)(h->N / 4)));
@@ -1158,6 +1134,7 @@ int cvf3_create(const cvf_params* p, void* stream, void* dev_state, cvf3_handle*
                                h->stream));
   CREATE_CHECK(cudaMemcpyAsync(h->vol_dev, &va, sizeof(va), cudaMemcpyHostToDevice, h->stream));
   CREATE_CHECK(cudaMemsetAsync(h->ctrl, 0, sizeof(Ctrl), h->stream));
+  CREATE_CHECK(cudaMemsetAsync(h->rc_dev, 0, sizeof(unsigned long long) * 20, h->stream));
 
   Args3& A = h->args;
   A.state = h->state;
@@ -1276,14 +1253,12 @@ int cvf3_sweep(cvf3_handle* h, int64_t n_sweeps, int32_t record_every) {
 int cvf3_observables(cvf3_handle* h, cvf_obs* out) {
   NvtxRange nvtx_range("cvf3_observables");
   if (!h || !out) return set_error(CVF_EINVAL, "NULL argument");
-  CVF_CUDA_CHECK(cudaMemsetAsync(h->rc_dev, 0, sizeof(unsigned long long) * 10, h->stream));
-  k_count3<<<h->grid_count, kThreads3, 0, h->stream>>>(h->state, h->args.L, h->args.L2,
-                                                        h->args.N, h->args.div_L, h->args.div_L2,
-                                                        nullptr, h->rc_dev);
-  k_observables3<<<1, 32, 0, h->stream>>>(h->vol_dev, h->ctrl, h->rc_dev, h->obs_dev);
-  CVF_CUDA_CHECK(cudaGetLastError());
-  CVF_CUDA_CHECK(cudaMemcpyAsync(h->host_pinned, h->obs_dev, sizeof(cvf_obs),
-                                 cudaMemcpyDeviceToHost, h->stream));
+  ObserveArgs a;
+  a.item[0] = ObserveItem{h->state, h->N, h->vol_dev, h->ctrl, h->rc_dev + 10,
+                          reinterpret_cast<cvf_obs*>(h->host_pinned)};
+  a.error = nullptr;
+  a.error_out = nullptr;
+  CVF_CUDA_CHECK(launch_observe(a, 1, h->N, true, h->stream));
   CVF_CUDA_CHECK(cudaStreamSynchronize(h->stream));
   std::memcpy(out, h->host_pinned, sizeof(cvf_obs));
   return status_error(out->status);
@@ -1424,7 +1399,7 @@ int cvf3_recount(cvf3_handle* h, int64_t* n_hb_raw, int64_t* n_sigma) {
   CVF_CUDA_CHECK(cudaMemsetAsync(h->rc_dev, 0, sizeof(unsigned long long) * 10, h->stream));
   k_count3<<<h->grid_count, kThreads3, 0, h->stream>>>(h->state, h->args.L, h->args.L2,
                                                         h->args.N, h->args.div_L, h->args.div_L2,
-                                                        h->rc_dev + 8, nullptr);
+                                                        h->rc_dev + 8);
   CVF_CUDA_CHECK(cudaGetLastError());
   unsigned long long r[2];
   CVF_CUDA_CHECK(cudaMemcpyAsync(h->host_pinned, h->rc_dev + 8, sizeof(r), cudaMemcpyDeviceToHost,

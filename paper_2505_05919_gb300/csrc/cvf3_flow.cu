@@ -450,8 +450,6 @@ Flow3Plan flow3_plan(const Args3& A, bool cmp64) {
 cudaError_t launch_flow3(const Args3& A, const Flow3Plan& P, WaveHdr* H, long long n_steps,
                          int every, cudaStream_t s) {
   if (P.blocks < 1) return cudaErrorCooperativeLaunchTooLarge;
-  const cudaError_t e = cudaMemsetAsync(H, 0, sizeof(WaveHdr), s);
-  if (e != cudaSuccess) return e;
   uint32_t gpb = P.groups_per_block;
   uint32_t* copy = reinterpret_cast<uint32_t*>(H + 1);
   void* args[6] = {const_cast<Args3*>(&A), &gpb, &H, &copy, &n_steps, &every};

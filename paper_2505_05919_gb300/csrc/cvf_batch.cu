@@ -16,6 +16,7 @@
 #include "cvf_device.cuh"
 #include "cvf_host.h"
 #include "cvf_lattice.cuh"
+#include "cvf_observe.cuh"
 #include "cvf_tile.cuh"
 
 using namespace cvf;
@@ -123,8 +124,7 @@ struct cvf_batch {
   // device staging (records + histograms), a pinned copy of the records and
   // of the launch error word, and the event that marks the copy done
   struct ObsSlot {
-    cvf_obs* d_obs;
-    unsigned long long* d_hist;
+    unsigned long long* d_counts;  // ten words per record (ObserveItem)
     cvf_obs* h_obs;
     unsigned int* h_err;
     int cap;
@@ -375,15 +375,14 @@ int launch_error(unsigned int err) {
 // (Re)allocates a ticket slot's staging for cap records; the slot's last
 // copy must be done.
 cudaError_t grow_obs_slot(cvf_batch::ObsSlot& o, int cap) {
-  if (o.d_obs) cudaFree(o.d_obs);
-  if (o.d_hist) cudaFree(o.d_hist);
+  if (o.d_counts) cudaFree(o.d_counts);
   if (o.h_obs) cudaFreeHost(o.h_obs);
-  o.d_obs = nullptr;
-  o.d_hist = nullptr;
+  o.d_counts = nullptr;
   o.h_obs = nullptr;
   o.cap = 0;
-  cudaError_t e = cudaMalloc(&o.d_obs, sizeof(cvf_obs) * cap);
-  if (e == cudaSuccess) e = cudaMalloc(&o.d_hist, sizeof(unsigned long long) * 9 * cap);
+  const size_t bytes = sizeof(unsigned long long) * 10 * cap;
+  cudaError_t e = cudaMalloc(&o.d_counts, bytes);
+  if (e == cudaSuccess) e = cudaMemset(o.d_counts, 0, bytes);
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&o.h_obs), sizeof(cvf_obs) * cap);
   if (e == cudaSuccess) o.cap = cap;
   return e;
@@ -690,23 +689,30 @@ int cvf_batch_observables_enqueue(cvf_batch* b, const int32_t* replicas, int32_t
     while (cap < n) cap *= 2;
     CVF_CUDA_CHECK(grow_obs_slot(o, cap));
   }
-  if (n > 0) {
-    CVF_CUDA_CHECK(cudaMemsetAsync(o.d_hist, 0, sizeof(unsigned long long) * 9 * n, b->stream));
-    for (int i = 0; i < n; ++i) {
-      const Replica& r = b->reps[replicas[i]];
-      const int grid = (int)std::max<long long>(1, std::min<long long>((r.N + kThreads - 1) / kThreads, 2048));
-      k_histogram<<<grid, kThreads, 0, b->stream>>>(r.state + (size_t)(r.sweep_host & 1) * r.N, r.N,
-                                                    o.d_hist + 9 * i);
-      k_observables<<<1, 32, 0, b->stream>>>(r.vol, r.ctrl, o.d_hist + 9 * i, o.d_obs + i);
-    }
-    CVF_CUDA_CHECK(cudaGetLastError());
-    CVF_CUDA_CHECK(cudaMemcpyAsync(o.h_obs, o.d_obs, sizeof(cvf_obs) * n, cudaMemcpyDeviceToHost,
-                                   b->stream));
-  }
+  // the records (and, with the first, the last launch's error word) go to the
+  // pinned slot from the kernel; kObserveItems replicas per launch
   o.h_err[0] = 0;
-  if (b->d_work)
-    CVF_CUDA_CHECK(cudaMemcpyAsync(o.h_err, reinterpret_cast<char*>(b->d_work) + offsetof(BatchWork, error),
-                                   sizeof(unsigned int), cudaMemcpyDeviceToHost, b->stream));
+  const unsigned int* err = b->d_work ? reinterpret_cast<const unsigned int*>(
+                                            reinterpret_cast<char*>(b->d_work) +
+                                            offsetof(BatchWork, error))
+                                      : nullptr;
+  for (int i0 = 0; i0 < n; i0 += kObserveItems) {
+    ObserveArgs a;
+    const int m = std::min(kObserveItems, n - i0);
+    long long most = 0;
+    for (int k = 0; k < m; ++k) {
+      const Replica& r = b->reps[replicas[i0 + k]];
+      a.item[k] = ObserveItem{r.state + (size_t)(r.sweep_host & 1) * r.N, r.N, r.vol, r.ctrl,
+                              o.d_counts + 10 * (i0 + k), o.h_obs + i0 + k};
+      most = std::max(most, r.N);
+    }
+    a.error = err;
+    a.error_out = (i0 == 0) ? o.h_err : nullptr;
+    CVF_CUDA_CHECK(launch_observe(a, m, most, false, b->stream));
+  }
+  if (n == 0 && err)
+    CVF_CUDA_CHECK(cudaMemcpyAsync(o.h_err, err, sizeof(unsigned int), cudaMemcpyDeviceToHost,
+                                   b->stream));
   CVF_CUDA_CHECK(cudaEventRecord(o.ev, b->stream));
   o.n = n;
   o.ticket = t;
@@ -752,12 +758,20 @@ int cvf_batch_get_state(cvf_batch* b, int32_t replica, uint16_t* host, size_t n)
   const Replica& r = b->reps[replica];
   if (!host || (long long)n != r.N)
     return set_error(CVF_EINVAL, "n=%zu, replica %d has %lld cells", n, replica, r.N);
-  rc = batch_status(b);
-  if (rc) return rc;
+  // the state and the last launch's error word behind one synchronisation
+  // (256 replicas of 32^2 to 512^2: a wait each for the launch, the word and the
+  // state took half of the read-back)
+  std::memset(b->h_pinned, 0, sizeof(unsigned int));
+  if (b->d_work)
+    CVF_CUDA_CHECK(cudaMemcpyAsync(b->h_pinned,
+                                   reinterpret_cast<char*>(b->d_work) + offsetof(BatchWork, error),
+                                   sizeof(unsigned int), cudaMemcpyDeviceToHost, b->stream));
   CVF_CUDA_CHECK(cudaMemcpyAsync(host, r.state + (size_t)(r.sweep_host & 1) * r.N,
                                  sizeof(uint16_t) * n, cudaMemcpyDeviceToHost, b->stream));
   CVF_CUDA_CHECK(cudaStreamSynchronize(b->stream));
-  return CVF_OK;
+  unsigned int err = 0;
+  std::memcpy(&err, b->h_pinned, sizeof(err));
+  return launch_error(err);
 }
 
 int cvf_batch_memory(cvf_batch* b, uint64_t* reserved, uint64_t* used) {
@@ -788,8 +802,7 @@ int cvf_batch_destroy(cvf_batch* b) {
   }
   for (int k = 0; k < kObsSlots; ++k) {
     cvf_batch::ObsSlot& o = b->obs[k];
-    if (o.d_obs) cudaFree(o.d_obs);
-    if (o.d_hist) cudaFree(o.d_hist);
+    if (o.d_counts) cudaFree(o.d_counts);
     if (o.h_obs) cudaFreeHost(o.h_obs);
     if (o.h_err) cudaFreeHost(o.h_err);
     if (o.ev) cudaEventDestroy(o.ev);

@@ -271,6 +271,14 @@ __device__ __forceinline__ void flow_books(const ARGS& A, VolumeArgs& V, WaveHdr
     wave_engine(A.ctrl, V, A.keys, H, step0, n_steps);
   else if (threadIdx.x < 96)
     flow_commit(A.ctrl, V, A.ring, A.ring_cap, every, H, blocks, tag, end_tag, step0, n_steps);
+  if (threadIdx.x >= 96) return;
+  // every clerk has reported the last step and looks at the header no more: it is
+  // left as the next launch wants it (an abandoned launch leaves it as it is)
+  asm volatile("bar.sync 6, 96;" ::: "memory");
+  if (*(volatile unsigned int*)&H->abort) return;
+  uint4* const words = reinterpret_cast<uint4*>(H);
+  for (int i = threadIdx.x; i < (int)(sizeof(WaveHdr) / 16); i += 96)
+    words[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // The blocks of `fn` that fit the GPU at once.

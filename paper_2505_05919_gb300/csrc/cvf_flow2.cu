@@ -529,8 +529,6 @@ Flow2Plan flow2_plan(int L, int schedule, int rng_words, bool cmp64) {
 cudaError_t launch_flow2(const LatticeArgs& A, const Flow2Plan& P, WaveHdr* H, long long n_steps,
                          int every, cudaStream_t s) {
   uint32_t* copy = reinterpret_cast<uint32_t*>(H + 1);
-  const cudaError_t e = cudaMemsetAsync(H, 0, sizeof(WaveHdr), s);
-  if (e != cudaSuccess) return e;
   void* args[6] = {const_cast<LatticeArgs*>(&A), const_cast<Flow2Geom*>(&P.geom), &H, &copy,
                    &n_steps, &every};
   return cudaLaunchCooperativeKernel(P.kernel, dim3(P.blocks + 1), dim3(P.threads), args, 0, s);

@@ -16,6 +16,7 @@
 #include "cvf_flow2.cuh"
 #include "cvf_host.h"
 #include "cvf_lattice.cuh"
+#include "cvf_observe.cuh"
 #include "cvf_tile.cuh"
 #include "cvf_tma.cuh"
 #include <cudaTypedefs.h>
@@ -123,18 +124,6 @@ __global__ void k_volume_prologue(const VolumeArgs* __restrict__ V, Ctrl* ctl, R
   }
 }
 
-__global__ void k_observables(const VolumeArgs* __restrict__ V, const Ctrl* ctl,
-                              const unsigned long long* hist, cvf_obs* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    Ctrl c = *ctl;
-    if (hist) c.n_coop = (long long)hist[8];  // counted now from the lattice
-    cvf_obs o = make_obs(*V, &c);
-    if (hist)
-      for (int v = 0; v < 8; ++v) o.n_state[v] = (long long)hist[v];
-    *out = o;
-  }
-}
-
 // The first word of w[0, n) that is not a valid cell for q (a spare bit set or
 // an arm >= q), as an atomic minimum into *first (left at its initial value,
 // the caller's all-ones, when every word is valid).
@@ -148,34 +137,6 @@ __global__ void __launch_bounds__(kThreads) k_first_invalid(const uint16_t* __re
         ((x >> 12) & 7u) >= q)
       atomicMin(first, (unsigned long long)i);
   }
-}
-
-// N_q' of a lattice (the number of sigma variables in each state) added to
-// out[0..8), and its equal in-cell pairs (N_sigma) added to out[8].
-__global__ void __launch_bounds__(kThreads) k_histogram(const uint16_t* __restrict__ state,
-                                                        long long N, unsigned long long* out) {
-  __shared__ unsigned long long s_cnt[9];
-  if (threadIdx.x < 9) s_cnt[threadIdx.x] = 0;
-  __syncthreads();
-  uint32_t c[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  uint32_t pairs = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
-       i += (long long)gridDim.x * blockDim.x) {
-    const uint32_t w = state[i];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const uint32_t v = (w >> (4 * a)) & 7u;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) c[k] += (v == (uint32_t)k) ? 1u : 0u;
-    }
-    pairs += cell_pairs(w);
-  }
-#pragma unroll
-  for (int k = 0; k < 8; ++k)
-    if (c[k]) atomicAdd(&s_cnt[k], (unsigned long long)c[k]);
-  if (pairs) atomicAdd(&s_cnt[8], (unsigned long long)pairs);
-  __syncthreads();
-  if (threadIdx.x < 9 && s_cnt[threadIdx.x]) atomicAdd(&out[threadIdx.x], s_cnt[threadIdx.x]);
 }
 
 // ---------------------------------------------------------------------------
@@ -633,12 +594,11 @@ struct cvf_handle {
   cvf_obs* ring;
   long long ring_cap;
   long long ring_tail;
-  cvf_obs* obs_dev;
   unsigned long long* table_dev;     // [2][24] (dN_HB+1)*8 + dN_sigma+3
   bool cmp64;                        // some threshold is 0: compare in 64 bits
   long long sweep_host;              // steps enqueued so far: buffer sweep & 1 is current
   VolumeArgs* vol_dev;
-  unsigned long long* rc_dev;
+  unsigned long long* rc_dev;        // ten words of scratch, then ten of k_observe
   void* host_pinned;
   LatticeArgs args;
   CUtensorMap tm[2];  // TMA descriptors of the two halves of the state pair
@@ -673,7 +633,6 @@ void release(cvf_handle* h) {
   if (h->own_state && h->state) cudaFree(h->state);
   if (h->ctrl) cudaFree(h->ctrl);
   if (h->ring) cudaFree(h->ring);
-  if (h->obs_dev) cudaFree(h->obs_dev);
   if (h->table_dev) cudaFree(h->table_dev);
   if (h->vol_dev) cudaFree(h->vol_dev);
   if (h->rc_dev) cudaFree(h->rc_dev);
@@ -1020,10 +979,9 @@ int cvf_create(const cvf_params* p, void* stream, void* dev_state, cvf_handle** 
   }
   CREATE_CHECK(cudaMalloc(&h->ctrl, sizeof(Ctrl)));
   CREATE_CHECK(cudaMalloc(&h->ring, sizeof(cvf_obs) * (size_t)h->ring_cap));
-  CREATE_CHECK(cudaMalloc(&h->obs_dev, sizeof(cvf_obs)));
   CREATE_CHECK(cudaMalloc(&h->table_dev, sizeof(unsigned long long) * 48));
   CREATE_CHECK(cudaMalloc(&h->vol_dev, sizeof(VolumeArgs)));
-  CREATE_CHECK(cudaMalloc(&h->rc_dev, sizeof(unsigned long long) * 9));
+  CREATE_CHECK(cudaMalloc(&h->rc_dev, sizeof(unsigned long long) * 20));
   CREATE_CHECK(cudaMallocHost(&h->host_pinned, 4096));
 
   unsigned long long table24[48];
@@ -1034,6 +992,7 @@ int cvf_create(const cvf_params* p, void* stream, void* dev_state, cvf_handle** 
                                h->stream));
   CREATE_CHECK(cudaMemcpyAsync(h->vol_dev, &va, sizeof(va), cudaMemcpyHostToDevice, h->stream));
   CREATE_CHECK(cudaMemsetAsync(h->ctrl, 0, sizeof(Ctrl), h->stream));
+  CREATE_CHECK(cudaMemsetAsync(h->rc_dev, 0, sizeof(unsigned long long) * 20, h->stream));
 
   h->args.state = h->state;
   h->args.ctrl = h->ctrl;
@@ -1143,12 +1102,12 @@ int cvf_sweep(cvf_handle* h, int64_t n_sweeps, int32_t record_every) {
 int cvf_observables(cvf_handle* h, cvf_obs* out) {
   NvtxRange nvtx_range("cvf_observables");
   if (!h || !out) return set_error(CVF_EINVAL, "NULL argument");
-  CVF_CUDA_CHECK(cudaMemsetAsync(h->rc_dev, 0, sizeof(unsigned long long) * 9, h->stream));
-  k_histogram<<<h->grid_cells, kThreads, 0, h->stream>>>(current(h), h->N, h->rc_dev);
-  k_observables<<<1, 32, 0, h->stream>>>(h->vol_dev, h->ctrl, h->rc_dev, h->obs_dev);
-  CVF_CUDA_CHECK(cudaGetLastError());
-  CVF_CUDA_CHECK(cudaMemcpyAsync(h->host_pinned, h->obs_dev, sizeof(cvf_obs),
-                                 cudaMemcpyDeviceToHost, h->stream));
+  ObserveArgs a;
+  a.item[0] = ObserveItem{current(h), h->N, h->vol_dev, h->ctrl, h->rc_dev + 10,
+                          reinterpret_cast<cvf_obs*>(h->host_pinned)};
+  a.error = nullptr;
+  a.error_out = nullptr;
+  CVF_CUDA_CHECK(launch_observe(a, 1, h->N, false, h->stream));
   CVF_CUDA_CHECK(cudaStreamSynchronize(h->stream));
   std::memcpy(out, h->host_pinned, sizeof(cvf_obs));
   return status_error(out->status);
@@ -1329,7 +1288,7 @@ constexpr size_t kNoAllocScratchBytes = 64 * 1024;
 
 struct NoAllocScratch {
   Ctrl ctrl;
-  unsigned long long hist[9];
+  unsigned long long counts[10];  // k_observe's
   unsigned long long table24[48];
   VolumeArgs vol;
   cvf_obs obs;
@@ -1494,11 +1453,13 @@ extern "C" int cvf_sweep_noalloc(const cvf_params* p, void* dev_state, double V_
       tile_count(p->L, tile) >= resident_sweep_blocks(cmp64, p->rng_words, tile);
   for (int64_t i = 0; i < n_sweeps; ++i)
     CVF_CUDA_CHECK(launch_sweep(fn, grid, st, A, no_map, no_map, programmatic));
-  CVF_CUDA_CHECK(cudaMemsetAsync(s->hist, 0, sizeof(s->hist), st));
-  k_histogram<<<grid_cells, kThreads, 0, st>>>(A.state + (size_t)((sweep + n_sweeps) & 1) * N, N,
-                                               s->hist);
-  k_observables<<<1, 32, 0, st>>>(&s->vol, &s->ctrl, s->hist, &s->obs);
-  CVF_CUDA_CHECK(cudaGetLastError());
+  CVF_CUDA_CHECK(cudaMemsetAsync(s->counts, 0, sizeof(s->counts), st));
+  ObserveArgs oa;
+  oa.item[0] = ObserveItem{A.state + (size_t)((sweep + n_sweeps) & 1) * N, N, &s->vol, &s->ctrl,
+                           s->counts, &s->obs};
+  oa.error = nullptr;
+  oa.error_out = nullptr;
+  CVF_CUDA_CHECK(launch_observe(oa, 1, N, false, st));
   CVF_CUDA_CHECK(cudaMemcpyAsync(host_obs, &s->obs, sizeof(cvf_obs), cudaMemcpyDeviceToHost, st));
   if (records > 0)
     CVF_CUDA_CHECK(cudaMemcpyAsync(host_series, s->ring, sizeof(cvf_obs) * records,

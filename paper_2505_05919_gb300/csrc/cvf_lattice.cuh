@@ -42,8 +42,7 @@ struct LatticeArgs {
   int32_t use_tma;                   // 1: interior tiles are staged by TMA
 };
 
-// Kernels of cvf_lattice.cu that the batch reuses for initialisation and
-// observables.
+// Kernels of cvf_lattice.cu that the batch and the cubic lattice reuse.
 __global__ void k_init(uint16_t* __restrict__ state, int32_t L, uint32_t q, int random,
                        RoundKeys K);
 __global__ void k_recount(const uint16_t* __restrict__ base, int32_t L, const Ctrl* ctl,
@@ -53,10 +52,6 @@ __global__ void k_set_ctrl(const VolumeArgs* __restrict__ V, Ctrl* ctl, double V
                            long long sweep, long long N);
 __global__ void k_set_record(Ctrl* ctl, int record_every);
 __global__ void k_volume_prologue(const VolumeArgs* __restrict__ V, Ctrl* ctl, RoundKeys K);
-__global__ void k_observables(const VolumeArgs* __restrict__ V, const Ctrl* ctl,
-                              const unsigned long long* hist, cvf_obs* out);
-__global__ void k_histogram(const uint16_t* __restrict__ state, long long N,
-                            unsigned long long* out);
 
 // The resident sweep (cvf_resident2.cu): a square lattice of side L (a
 // multiple of kResCtas, 2 kResCtas <= L <= kResMaxSide) held in the shared

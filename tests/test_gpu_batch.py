@@ -228,3 +228,18 @@ def test_batch_two_word_draws_every_block_size(cfg):
         s, o = _solo(p, [steps[i]])
         assert np.array_equal(got[i][0], s), (cfg, i)
         _same(got[i][1], o)
+
+
+def test_observables_of_many_replicas():
+    # more records than one launch takes, sides from one block's single load up,
+    # each against the counts of the state itself
+    sides = [2, 4, 6, 10, 32, 66, 130] * 10
+    with Batch([_params(L, seed=300 + i, q=2 + i % 7) for i, L in enumerate(sides)]) as b:
+        b.sweep([1 + i % 5 for i in range(len(sides))])
+        got = b.observables_many(list(range(len(sides))))
+        for i, L in enumerate(sides):
+            s = b.state(i).reshape(-1).astype(np.int64)
+            arms = np.stack([(s >> (4 * a)) & 7 for a in range(4)], 1)
+            assert list(got[i]["n_state"]) == [int((arms == v).sum()) for v in range(8)], i
+            pairs = sum(int((arms[:, x] == arms[:, y]).sum()) for x in range(4) for y in range(x))
+            assert got[i]["n_coop"] == pairs and got[i]["status"] == 0, i
