@@ -23,7 +23,7 @@
 // (0.27 to 0.5 us between SMs), the four arm updates -- up to about 512^2, the
 // instructions of the cells beyond (the launches and waits that it replaces
 // took 2.7 us per step at 64^2, 8.2 at 258^2, 7.3 at 512^2 and 11.9 at 1024^2;
-// now 1.8, 1.9, 2.7 and 7.6).  The draws of a part are made before its first
+// now 1.3, 1.9, 2.7 and 7.6).  The draws of a part are made before its first
 // load.
 #include <cuda_runtime.h>
 
@@ -251,6 +251,164 @@ __global__ void __launch_bounds__(NT + 32, 1)
       if ((uint32_t)k < h && dcheck((y0 + k) * Lh + p < L * Lh, err, kSiteTileWrite))
         dst[(y0 + k) * Lh + p] = w[k];
   }
+}
+
+// ---------------------------------------------------------------------------
+// Small lattices: the same with one word per thread in the shared memory of a
+// thread-block cluster.  A CTA holds a run of words and, on either side, copies
+// of the Lh words next to it (a word's neighbours are at most Lh away), which
+// their owners write as well: every thread reads its own CTA's memory only, so
+// a part costs a store to the next SM and not a load's round trip to it (64^2:
+// 1.27 us per step against 1.41 with remote loads and 1.77 through L2).  The
+// last CTA of the cluster runs the volume engine and the committer on an SM of
+// its own (FP64 instructions hold back the integer multiplies beside them).  The
+// words live in shared memory for one call only, so their tags start at 0.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
+}
+// The address of shared-memory word p in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const uint32_t* p, uint32_t rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;"
+      : "=r"(a)
+      : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t v) {
+  asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+constexpr int kClusterThreads = 576;  // sweeping threads of a CTA
+constexpr int kClusterHalo = 64;      // words of a row at most
+
+template <int RNG_WORDS, bool CMP64>
+__global__ void __launch_bounds__(kClusterThreads + 32, 1)
+    k_flow2_cluster(const __grid_constant__ LatticeArgs A, const __grid_constant__ Flow2Geom G,
+                    WaveHdr* H, long long n_steps, int every) {
+  __shared__ union {
+    Flow2Smem sweep;
+    VolumeArgs vol;
+  } U;
+  __shared__ uint32_t s_word[kClusterThreads + 2 * kClusterHalo];
+  __shared__ uint32_t s_no_tag;
+  Ctrl* const ctl = A.ctrl;
+  unsigned int* const err = &ctl->error;
+  const long long step0 = *(volatile long long*)&ctl->sweep;  // (as in k_flow2)
+  const uint32_t L = (uint32_t)A.L, Lh = L >> 1, q = A.q;
+  const long long N = (long long)L * L;
+  const bool books = blockIdx.x == gridDim.x - 1u;
+  Flow2Smem& S = U.sweep;
+  const uint32_t t_lo = blockIdx.x * G.per_block, t_hi = min(t_lo + G.per_block, G.items);
+  const int warps = books ? 0 : (int)((t_hi - t_lo + 31u) / 32u);
+  const bool sweeps = threadIdx.x < kClusterThreads && (int)(threadIdx.x >> 5) < warps;
+  const bool mine = sweeps && t_lo + threadIdx.x < t_hi;
+  const uint32_t item = sweeps ? min(t_lo + threadIdx.x, t_hi - 1u) : 0u;
+  const uint32_t y = fdiv(item, G.div_row), p = item - y * Lh;
+  // the CTA's words lie at s_word[Lh], those before and after them around
+  const int cnt = (int)(t_hi - t_lo), W = (int)G.items;
+  auto word_of = [&](uint32_t i) -> volatile uint32_t* {
+    int d = (int)i - (int)t_lo;
+    if (d < 0 || d >= cnt) {
+      const int before = (d < 0) ? d : d - W;
+      d = (before >= -(int)Lh) ? before : (d < 0) ? d + W : d;
+    }
+    if (!dcheck(d >= -(int)Lh && d < cnt + (int)Lh, err, kSiteResident2)) d = 0;
+    return s_word + (int)Lh + d;
+  };
+  volatile uint32_t *own = s_word, *up = s_word, *down = s_word, *left = s_word, *right = s_word;
+  uint32_t to_prev = 0u, to_next = 0u;  // the word's copies in the CTAs beside this one
+  if (sweeps) {
+    own = word_of(item);
+    up = word_of(((y == 0u) ? L - 1u : y - 1u) * Lh + p);
+    down = word_of(((y + 1u == L) ? 0u : y + 1u) * Lh + p);
+    left = word_of(y * Lh + ((p == 0u) ? Lh - 1u : p - 1u));
+    right = word_of(y * Lh + ((p + 1u == Lh) ? 0u : p + 1u));
+    const uint32_t n = gridDim.x - 1u;  // CTAs with words
+    if (n > 1u && mine) {
+      const uint32_t prev = (blockIdx.x == 0u) ? n - 1u : blockIdx.x - 1u;
+      const uint32_t next = (blockIdx.x + 1u == n) ? 0u : blockIdx.x + 1u;
+      const uint32_t prev_cnt = min(G.per_block, G.items - prev * G.per_block);
+      if (item - t_lo < Lh) to_prev = cluster_addr(s_word + Lh + prev_cnt + (item - t_lo), prev);
+      if (t_hi - item <= Lh) to_next = cluster_addr(s_word + Lh - (t_hi - item), next);
+    }
+  }
+  auto put = [&](uint32_t v) {
+    *own = v;
+    if (to_prev) st_cluster(to_prev, v);
+    if (to_next) st_cluster(to_next, v);
+  };
+  uint32_t w = 0u;
+  if (sweeps && dcheck(item < L * Lh, err, kSiteResident2))
+    w = __ldcg(reinterpret_cast<const uint32_t*>(A.state + (size_t)(step0 & 1) * N) + item);
+  if (!books) flow2_setup(S, A, kClusterThreads + 32);
+  cluster_sync_all();  // every CTA runs
+  if (mine) put(w);
+  __syncthreads();
+  cluster_sync_all();  // and every word is in place
+
+  auto sweep = [&]() {
+    const unsigned int full = 0xFFFFFFFFu;
+    for (long long rel = 0; rel < n_steps; ++rel) {
+      const long long step = step0 + rel;
+      FlowSlot& slot = S.ring[rel % kWaveRing];
+      const uint32_t tag = (uint32_t)((unsigned long long)rel & 0xFFFFFFu);
+      const StepDraw sd = step_draw((uint32_t)((unsigned long long)step & 0xFFFFFFFFu),
+                                    (uint32_t)((unsigned long long)step >> 32), A.keys);
+      uint32_t pk = 0;
+      int g = 0;
+#pragma unroll
+      for (int colour = 0; colour < 2; ++colour) {
+        const uint32_t hi = (y + (uint32_t)colour) & 1u;
+        const CellWords<RNG_WORDS> draw = cell_words<RNG_WORDS>(y * L + 2u * p + hi, sd, A.keys);
+        uint32_t acc[4], kk[4];
+        split_draws<RNG_WORDS>(draw.u, draw.p, q, acc, kk);
+        if (colour == 0) {
+          if (!flow_ready(slot, rel, H, err)) return;
+          g = slot.g;
+        }
+        const uint32_t need = tag_bits(tag + (uint32_t)colour, tag + (uint32_t)colour);
+        const uint32_t vertical = hi ? 0x880000u : 0x88u, across = hi ? 0x88u : 0x880000u;
+        uint32_t side, top, bottom;
+        for (unsigned int spins = 0;;) {
+          side = *(hi ? right : left);
+          top = *up;
+          bottom = *down;
+          const uint32_t late =
+              ((side ^ need) & across) | (((top ^ need) | (bottom ^ need)) & vertical);
+          if (__all_sync(full, late == 0u)) break;
+          if ((++spins & 1023u) == 0u && flow_stop(spins >> 2, H, err)) return;
+        }
+        if (mine) {
+          const uint32_t cell = update_cell<CMP64>(w, side, side, top, bottom, (int)hi, acc, kk, q,
+                                                   S.Tb[g], pk);
+          w = put_cell(w, cell, hi != 0u);
+          const uint32_t other = tag + (uint32_t)colour;
+          put(w | (hi ? tag_bits(other, tag + 1u) : tag_bits(tag + 1u, other)));
+        }
+      }
+      TileCounts cnt{0, 0, 0};
+      cnt.add(pk);
+      const bool rec = step_recorded(every, step);
+      uint32_t hist[4] = {0u, 0u, 0u, 0u};
+      if (rec && mine) {
+        const uint32_t n = count_word4(w & 0xFFFFu) + count_word4(w >> 16);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) hist[v] = (n >> (4 * v)) & 0x000F000Fu;
+      }
+      flow_report2(slot, cnt, rec, hist);
+    }
+    if (mine && dcheck(item < L * Lh, err, kSiteResident2))
+      reinterpret_cast<uint32_t*>(A.state + (size_t)((step0 + n_steps) & 1) * N)[item] = w;
+  };
+  if (books)
+    flow_books(A, U.vol, H, (int)gridDim.x - 1, &s_no_tag, 0u, step0, n_steps, every);
+  else if (sweeps)
+    sweep();
+  else if (threadIdx.x >= kClusterThreads)
+    flow_clerk([](long long) { return 0ull; }, S.ring, warps, H, err, step0, n_steps, every);
+  __syncwarp();
+  cluster_sync_all();  // no CTA leaves while another may still read its words
 }
 
 // ---------------------------------------------------------------------------
@@ -504,6 +662,65 @@ const Flow2Form kStrips[] = {{1, 480, flow2_kernel<1, 480>}, {1, 992, flow2_kern
 // with 480; 4096^2 195, 201, 240).
 const Flow2Form kLayerOne = {0, 480, flow2_layer_kernel<true, 480>};
 const Flow2Form kLayerMany = {0, 992, flow2_layer_kernel<false, 992>};
+// The cluster form: at most fifteen CTAs with words (128^2) and one with the
+// books; a CTA for every so many words (64^2 1.27 us per step with 64 or 128,
+// 1.30 with 256, 1.56 with 544).
+constexpr int kClusterCtas = 15, kClusterShare = 128;
+
+const void* cluster_kernel(int rng_words, bool cmp64) {
+  if (rng_words == 1)
+    return cmp64 ? (const void*)k_flow2_cluster<1, true> : (const void*)k_flow2_cluster<1, false>;
+  return cmp64 ? (const void*)k_flow2_cluster<2, true> : (const void*)k_flow2_cluster<2, false>;
+}
+
+cudaLaunchConfig_t cluster_config(int ctas, cudaLaunchAttribute* attr, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kClusterThreads + 32);
+  cfg.stream = s;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = ctas;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Adopts the cluster form if the lattice's words fit one cluster and the GPU can
+// place it.
+bool adopt_cluster(Flow2Plan* P, int rng_words, bool cmp64, long long words, long long row) {
+  if (row > kClusterHalo || words > (long long)kClusterCtas * kClusterThreads) return false;
+  // (the last CTA holds a row of words at least: a word then has copies in the
+  // CTAs beside its own only)
+  long long ctas = std::min<long long>(kClusterCtas, (words + kClusterShare - 1) / kClusterShare);
+  long long share = 0;
+  for (;; --ctas) {
+    share = ((words + ctas - 1) / ctas + 31) / 32 * 32;
+    ctas = (words + share - 1) / share;
+    if (ctas == 1 || words - (ctas - 1) * share >= row) break;
+  }
+  if (share > kClusterThreads) return false;
+  const void* const kernel = cluster_kernel(rng_words, cmp64);
+  const int n = (int)ctas + 1;  // + the books'
+  int clusters = 0;
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = cluster_config(n, &attr, nullptr);
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess || clusters < 1) {
+    cudaGetLastError();
+    return false;
+  }
+  P->kernel = kernel;
+  P->threads = kClusterThreads + 32;
+  P->blocks = n - 1;
+  P->cluster = true;
+  P->geom.items = (uint32_t)words;
+  P->geom.per_block = (uint32_t)share;
+  P->copy_words = 0;
+  return true;
+}
 
 }  // namespace
 
@@ -520,6 +737,7 @@ Flow2Plan flow2_plan(int L, int schedule, int rng_words, bool cmp64) {
   }
   const long long Lh = L / 2;
   P.geom.div_row = make_fastdiv((uint32_t)Lh);
+  if (adopt_cluster(&P, rng_words, cmp64, Lh * L, Lh)) return P;
   P.copy_words = (size_t)kFlow2Head + (size_t)(Lh * L);
   for (const Flow2Form& form : kStrips)
     if (adopt(&P, form, rng_words, cmp64, Lh * ((L + form.v - 1) / form.v), true)) break;
@@ -528,6 +746,13 @@ Flow2Plan flow2_plan(int L, int schedule, int rng_words, bool cmp64) {
 
 cudaError_t launch_flow2(const LatticeArgs& A, const Flow2Plan& P, WaveHdr* H, long long n_steps,
                          int every, cudaStream_t s) {
+  if (P.cluster) {
+    void* args[5] = {const_cast<LatticeArgs*>(&A), const_cast<Flow2Geom*>(&P.geom), &H, &n_steps,
+                     &every};
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = cluster_config(P.blocks + 1, &attr, s);
+    return cudaLaunchKernelExC(&cfg, P.kernel, args);
+  }
   uint32_t* copy = reinterpret_cast<uint32_t*>(H + 1);
   void* args[6] = {const_cast<LatticeArgs*>(&A), const_cast<Flow2Geom*>(&P.geom), &H, &copy,
                    &n_steps, &every};

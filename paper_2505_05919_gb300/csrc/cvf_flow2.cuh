@@ -23,6 +23,7 @@ struct Flow2Geom {
 struct Flow2Plan {
   const void* kernel;
   int threads, blocks;  // blocks 0: the lattice is too large for it
+  bool cluster;         // one cluster holds the words: no copy
   Flow2Geom geom;
   size_t copy_words;
 };

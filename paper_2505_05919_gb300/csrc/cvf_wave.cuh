@@ -171,20 +171,14 @@ __device__ inline void wave_engine(Ctrl* ctl, const VolumeArgs& sV, const RoundK
     wave_publish(H, 0, cur);
   }
   engine_sync();
-  // one thread: the ring has room for the move of relative step r
+  // one thread: waits until the ring has room for the move of relative step r (a
+  // step more than kWaveRing behind it is committed); `seen` is what it last saw
+  unsigned int seen = 0;
   auto room = [&](long long r) {
-    return r < kWaveRing ||
-           wave_wait_geq(&H->committed, (unsigned int)(r - kWaveRing + 1), H, err);
-  };
-  auto publish = [&](long long r) {  // T holds the move of relative step r
-    if (r >= n_steps) return true;   // the next call's first: stays in T
-    if (!room(r)) return false;
-    VolumeResult m;
-    m.V = T.V;
-    m.u = T.u;
-    m.g = T.g;
-    m.accepted = T.acc;
-    wave_publish(H, r, m);
+    const long long need = r - kWaveRing + 1;
+    if (need <= (long long)seen) return true;
+    if (!wave_wait_geq(&H->committed, (unsigned int)need, H, err)) return false;
+    seen = ld_acquire(&H->committed);
     return true;
   };
   int shells = 0;  // of the last pass's root, the guess of the next
@@ -209,7 +203,11 @@ __device__ inline void wave_engine(Ctrl* ctl, const VolumeArgs& sV, const RoundK
         T.g = res.g;
         T.acc = res.accepted;
         T.flip = 0;
-        T.go = publish(r) ? 1 : 0;
+        T.go = 1;
+        if (r < n_steps) {  // the next call's first move stays in T
+          T.go = room(r) ? 1 : 0;
+          if (T.go) wave_publish(H, r, res);
+        }
       }
       engine_sync();
       if (!T.go) return;
@@ -264,28 +262,45 @@ __device__ inline void wave_engine(Ctrl* ctl, const VolumeArgs& sV, const RoundK
       const bool flip = !hard && g_new != bg;
       const unsigned int A = __ballot_sync(full, node && !hard && !flip && met);
       const unsigned int U = __ballot_sync(full, node && flip);
-      double Vc = bV, uc = bu;
-      int nn = 1, j = 0;
-      bool go = true;
-      for (; j < kWaveTree && go && r + j <= n_steps; ++j) {
+      double Vc = bV, uc = bu, myV = bV, myu = bu;
+      int nn = 1, j = 0, ac = 0, mya = 0;
+      for (; j < kWaveTree && r + j <= n_steps; ++j) {
         const int i = nn - 1;
         if ((U >> i) & 1u) break;
-        const int a = (int)((A >> i) & 1u);
+        ac = (int)((A >> i) & 1u);
         const double Vi = __shfl_sync(full, Vn, i), ui = __shfl_sync(full, un, i);
-        if (a) {
+        if (ac) {
           Vc = Vi;
           uc = ui;
         }
-        if (lane == 0) {
-          T.V = Vc;
-          T.u = uc;
-          T.acc = a;
-          go = publish(r + j);
+        if (lane == j) {  // lane j publishes the move of relative step r + j
+          myV = Vc;
+          myu = uc;
+          mya = ac;
         }
-        go = __shfl_sync(full, go ? 1 : 0, 0) != 0;
-        nn = 2 * nn + a;
+        nn = 2 * nn + ac;
       }
+      // the pass's moves behind one fence (a release for each, and a look at the
+      // commits before each, held every small lattice at 1.5 us per step)
+      const int n = (int)min((long long)j, n_steps - r);
+      bool go = true;
+      if (lane == 0 && n > 0) go = room(r + n - 1);
+      go = __shfl_sync(full, go ? 1 : 0, 0) != 0;
+      WaveMove& m = H->vring[(r + lane) % kWaveRing];
+      if (go && lane < n) {
+        volatile WaveMove* vm = &m;
+        vm->V = myV;
+        vm->u = myu;
+        vm->g = bg;
+        vm->acc = mya;
+      }
+      __syncwarp();
+      fence_acq_rel_gpu();
+      if (go && lane < n) st_relaxed_u32(&m.tag, (unsigned int)(r + lane + 1));
       if (lane == 0) {
+        T.V = Vc;
+        T.u = uc;
+        if (j > 0) T.acc = ac;
         T.flip = (j < kWaveTree && r + j <= n_steps && ((U >> (nn - 1)) & 1u)) ? 1 : 0;
         T.settled = j;
         T.go = go ? 1 : 0;

@@ -611,7 +611,8 @@ def test_maximum_size_sampled_windows(L):
             assert np.array_equal(got, want), (x0, y0)
 
 
-# The dataflow sweep at its edges: one and many blocks, blocks whose last warp is
+# The dataflow sweep at its edges: one CTA of a cluster and several (up to 128^2),
+# the copy in global memory beyond, one and many blocks, blocks whose last warp is
 # partly empty, each strip height and block size at the sides where it begins or
 # ends (152 SMs), a last strip of two rows (L % 4 == 2), two-word draws, every q,
 # the 64-bit compare, gate flips, every step recorded; and the layered schedule's
@@ -621,6 +622,10 @@ DATAFLOW = [
     (10, 60, 1, 0, dict(q=2, rng_words=2)),
     (34, 30, 1, 0, dict(q=8)),
     (66, 20, 7, 0, dict(init=oracle.INIT_ORDERED, rng_words=2)),
+    (22, 40, 1, 0, dict(kT=1e-3)),
+    (126, 12, 1, 0, dict(q=7)),
+    (128, 12, 1, 0, dict(rng_words=2)),
+    (130, 12, 1, 0, dict(init=oracle.INIT_ORDERED)),
     (380, 6, 2, 0, {}),
     (382, 6, 1, 0, dict(rng_words=2)),
     (546, 4, 1, 0, dict(kT=1e-3)),
