@@ -51,11 +51,14 @@ constexpr int kMaxSide3 = 1024;
 // The dataflow sweep (cvf3_flow.cu) takes cubes of up to this many groups
 // (128^3): there it still beats four launches per step, us per MC step with
 // the eta update: 16^3 4.0 against 14.6, 32^3 4.0 / 15.7, 64^3 8.0 / 17.0,
-// 100^3 22.4 / 29.9, 128^3 43.5 / 48.2, but 144^3 61.1 / 58.0 and 260^3 375 /
-// 271 (odd sides, without eta: 51^3 5.7 / 16.0, 101^3 32.8 / 35.4, 127^3 58.9
-// / 57.7): it looks at every word's tag, and sixteen warps of an SM hide less
-// latency than the launches' thirty-two.
+// 100^3 22.4 / 29.9, 128^3 43.9 / 48.2, but 144^3 61.1 / 58.0 and 260^3 375 /
+// 271: it looks at every word's tag, and sixteen warps of an SM hide less
+// latency than the launches' thirty-two.  Without the eta update and with rows
+// that are no whole groups, where a word is a load of its own, up to 112^3
+// (51^3 5.7 / 16.0, 73^3 16.7 / 19.9, 97^3 26.2 / 33.4, 109^3 38.2 / 41.8, but
+// 115^3 45.5 / 43.6).
 constexpr uint32_t kFlowMaxGroups = 1u << 19;
+constexpr uint32_t kFlowMaxGroupsRagged = 112u * 112u * 112u / 4u;
 
 // ---------------------------------------------------------------------------
 // One launch of a step.  ALIGNED: L % 4 == 0, a group (four consecutive
@@ -1176,7 +1179,8 @@ int cvf3_create(const cvf_params* p, void* stream, void* dev_state, cvf3_handle*
   h->grid = (int)std::max<long long>(1, std::min<long long>(blocks, (long long)sm_count() * per_sm));
   h->resident = resident3_auto(A, h->cmp64);
   h->plan = flow3_plan(A, h->cmp64);
-  h->flow = h->plan.blocks > 0 && A.groups <= kFlowMaxGroups;
+  h->flow = h->plan.blocks > 0 &&
+            A.groups <= (h->aligned || A.eta ? kFlowMaxGroups : kFlowMaxGroupsRagged);
   if (h->flow) {
     const size_t bytes = sizeof(WaveHdr) + sizeof(uint32_t) * h->plan.copy_words;
     if (cudaMalloc(reinterpret_cast<void**>(&h->wave), bytes) != cudaSuccess) {

@@ -101,8 +101,16 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
   const uint32_t g_lo = b * groups_per_block, g_hi = min(g_lo + groups_per_block, A.groups);
   const uint32_t g_first = g_lo + threadIdx.x;
   const bool eta_on = A.eta != nullptr;
-  // warps that have a group
-  const int warps = (int)min((g_hi - g_lo + 31u) / 32u, (uint32_t)(kFlowThreads / 32));
+  // Every warp sweeps as many groups (but for the last ones): a warp with one
+  // less would spend that time on loads that wait for the others, which slows
+  // them (70^3 without eta moves 22.3 us per step, so 14.0; 97^3 38.1 / 26.2).
+  // From four rounds of aligned groups on the idle warps cost more (100^3 19.5
+  // us with all of them, 21.9 so).
+  const uint32_t rounds = (groups_per_block + kFlowThreads - 1u) / kFlowThreads;
+  const uint32_t stride = (ALIGNED && rounds > 3u)
+                              ? (uint32_t)kFlowThreads
+                              : (groups_per_block / 32u + rounds - 1u) / rounds * 32u;
+  const int warps = (int)min((g_hi - g_lo + 31u) / 32u, stride / 32u);  // that have a group
   const uint32_t q = A.q;
   for (int g = 0; g < 2; ++g) fill_rows3(S.Tb[g], A.table + g * kRows3, kFlowBlock);
   fill_prop3(S.Tb[0], q, kFlowBlock);
@@ -182,7 +190,7 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
   };
 
   uint32_t xyz[4] = {0u, 0u, 0u, 0u}, w[4] = {0u, 0u, 0u, 0u}, cfg = 0u;
-  for (uint32_t gi = g_first; gi < g_hi; gi += kFlowThreads) {
+  for (uint32_t gi = g_first; gi < g_hi; gi += stride) {
     load_own(gi, A.state, w);
     store_own(gi, w, tag0 << 24);
     if (eta_on) {  // as many cubes as groups
@@ -223,7 +231,7 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
       // edges leaving the matching become allowed and those entering it
       // forbidden, so dN_HB = |bonded & old| - |bonded & new|.
       const uint32_t need = tag << 24;
-      for (uint32_t cube0 = g_lo + (threadIdx.x & ~31u); cube0 < g_hi; cube0 += kFlowThreads) {
+      for (uint32_t cube0 = g_lo + (threadIdx.x & ~31u); cube0 < g_hi; cube0 += stride) {
         const uint32_t cube = cube0 + (threadIdx.x & 31u);
         const bool mine = cube < g_hi;
         const Words4 r = philox(cube, s_lo, s_hi, kTagEta, A.keys);
@@ -289,7 +297,7 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
             wrp[p] = plus ? A.N : 0u - A.N;
           }
         }
-        for (uint32_t gi0 = g_lo + (threadIdx.x & ~31u); gi0 < g_hi; gi0 += kFlowThreads) {
+        for (uint32_t gi0 = g_lo + (threadIdx.x & ~31u); gi0 < g_hi; gi0 += stride) {
           const uint32_t gi = gi0 + (threadIdx.x & 31u);
           const bool mine = gi < g_hi;
           const uint32_t c0 = 4u * min(gi, g_hi - 1u);

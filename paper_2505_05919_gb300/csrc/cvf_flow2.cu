@@ -439,7 +439,10 @@ __global__ void __launch_bounds__(NT + 32, 1)
   Flow2Smem& S = U.sweep;
   uint32_t* const F = copy + kFlow2Head;
   const uint32_t t_lo = (blockIdx.x - 1u) * G.per_block, t_hi = min(t_lo + G.per_block, G.items);
-  const int warps = (int)min((t_hi - t_lo + 31u) / 32u, (uint32_t)(NT / 32));
+  // as many groups for every warp, as in the cubic sweep
+  const uint32_t rounds = (G.per_block + NT - 1u) / NT;
+  const uint32_t stride = (G.per_block / 32u + rounds - 1u) / rounds * 32u;
+  const int warps = (int)min((t_hi - t_lo + 31u) / 32u, stride / 32u);
   flow2_setup(S, A, NT + 32);
   __syncthreads();
   if (threadIdx.x >= NT) {
@@ -470,7 +473,7 @@ __global__ void __launch_bounds__(NT + 32, 1)
   CellWords<RNG_WORDS> draw[4];
   {
     const uint16_t* src = A.state + (size_t)(step0 & 1) * N;
-    for (uint32_t i0 = first; i0 < t_hi; i0 += NT) {
+    for (uint32_t i0 = first; i0 < t_hi; i0 += stride) {
       const uint32_t i = min(i0 + lane, t_hi - 1u);
       const Group gr = locate(i);
 #pragma unroll
@@ -509,7 +512,7 @@ __global__ void __launch_bounds__(NT + 32, 1)
       const bool last = j == nseg - 1;
       const uint32_t need = (tag + (uint32_t)j) << 16;
       const uint32_t out = (last ? tag + 4u : tag + 1u + (uint32_t)j) << 16;
-      for (uint32_t i0 = first; i0 < t_hi; i0 += NT) {
+      for (uint32_t i0 = first; i0 < t_hi; i0 += stride) {
         const bool mine = i0 + lane < t_hi;
         const Group gr = locate(min(i0 + lane, t_hi - 1u));
         uint32_t* const own = F + (size_t)gr.y * pitch + 4u * gr.x;

@@ -330,7 +330,8 @@ def test_lattice3_eta_every_step(T, P, init):
 
 # The dataflow sweep at its edges: blocks whose last warp is partly empty, the
 # last side with one group per thread and the first with several (51 / 52), rows
-# that groups cross (L % 4 != 0) with and without eta moves, one block, the
+# that groups cross (L % 4 != 0) with and without eta moves, several groups for
+# some of a block's warps and for all of them (70, 92, 100), one block, the
 # 64-bit compare, gate flips, every step recorded.
 FLOW = [
     (2, 1, 60, 1, {}),
@@ -344,6 +345,9 @@ FLOW = [
     (52, 1, 6, 1, {}),
     (54, 1, 5, 0, dict(q=3)),
     (61, 0, 4, 1, dict(kT=1e-3)),
+    (70, 0, 3, 1, {}),
+    (92, 1, 2, 1, {}),
+    (100, 0, 2, 1, dict(q=5)),
     (12, 1, 300, 1, dict(gates=True)),
     (33, 0, 120, 1, dict(gates=True)),
 ]
