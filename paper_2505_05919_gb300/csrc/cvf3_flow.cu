@@ -89,7 +89,7 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
   const uint32_t tag0 = *(volatile uint32_t*)copy + 8u;
   const uint32_t end_tag = tag0 + 8u * (uint32_t)((unsigned long long)n_steps & 0xFFFFFFu);
   if (blockIdx.x == 0) {
-    flow_books(A, U.vol, H, (int)gridDim.x - 1, copy, end_tag, step0, n_steps, every);
+    flow_books(A, U.vol, H, (int)gridDim.x - 1, copy, end_tag, step0, n_steps, every, err);
     return;
   }
   constexpr int kFlowThreads = ONE ? kFlowThreadsOne : kFlowThreadsMany;

@@ -14,6 +14,7 @@
 #include "cvf.h"
 #include "cvf_batch_kernel.cuh"
 #include "cvf_device.cuh"
+#include "cvf_flow2.cuh"
 #include "cvf_host.h"
 #include "cvf_lattice.cuh"
 #include "cvf_observe.cuh"
@@ -134,6 +135,8 @@ struct cvf_batch {
   } obs[kObsSlots];
   long long next_ticket;
   void* h_pinned;     // 4096 bytes
+  void* flow_mem;     // scratch of the dataflow launches (null: no room for it)
+  int flow_slots[2][kFlow2BatchForms];  // their resident blocks [cmp64][form], 0: not asked yet
   cudaGraphExec_t graph[kNumTileConfigs][2];  // [config][cmp64]
   int graph_n_reps[kNumTileConfigs][2];
   void* graph_work[kNumTileConfigs][2];
@@ -357,6 +360,39 @@ int launch(cvf_batch* b, int cfg, bool cmp64, int n_reps, int n_active) {
   return CVF_OK;
 }
 
+// The call as one dataflow launch, if its replicas' blocks are resident at once;
+// *done tells.
+int flow_sweep(cvf_batch* b, const std::vector<int32_t>& act, const int64_t* sweeps, bool cmp64,
+               bool* done) {
+  *done = false;
+  const int n = (int)act.size();
+  if (!b->flow_mem || n > kFlow2BatchMax || sweeps[act[0]] > (1ll << 30)) return CVF_OK;
+  int sides[kFlow2BatchMax], form = 0;
+  for (int i = 0; i < n; ++i) sides[i] = b->reps[act[i]].p.L;
+  Flow2Batch B;
+  if (!flow2_batch_plan(&B, sides, n, b->rng_words, cmp64, b->flow_slots[cmp64 ? 1 : 0], &form)) return CVF_OK;
+  B.err = &reinterpret_cast<BatchWork*>(b->d_work)->error;
+  for (int i = 0; i < n; ++i) {
+    const Replica& r = b->reps[act[i]];
+    LatticeArgs& a = B.item[i].args;
+    a = LatticeArgs{};
+    a.state = r.state;
+    a.ctrl = r.ctrl;
+    a.table24 = r.table;
+    a.vol = r.vol;
+    a.ring = r.ring;
+    a.ring_cap = kReplicaRingCap;
+    a.keys = make_round_keys(r.p.seed);
+    a.L = r.p.L;
+    a.q = (uint32_t)r.p.q;
+    B.item[i].n_steps = sweeps[act[i]];
+  }
+  CVF_CUDA_CHECK(cudaMemsetAsync(B.err, 0, sizeof(unsigned int), b->stream));
+  CVF_CUDA_CHECK(launch_flow2_batch(&B, b->flow_mem, b->rng_words, cmp64, form, b->stream));
+  *done = true;
+  return CVF_OK;
+}
+
 int check_replica(cvf_batch* b, int32_t id) {
   if (!b) return set_error(CVF_EINVAL, "batch is NULL");
   if (id < 0 || id >= (int)b->reps.size() || !b->reps[id].live)
@@ -429,6 +465,10 @@ int cvf_batch_create(const cvf_params* params, int32_t n, void* stream, cvf_batc
     if (e == cudaSuccess) e = cudaMemPoolSetAttribute(b->pool, cudaMemPoolAttrReleaseThreshold, &keep);
   }
   if (e == cudaSuccess) e = cudaMallocHost(&b->h_pinned, 4096);
+  if (e == cudaSuccess && cudaMalloc(&b->flow_mem, flow2_batch_scratch()) != cudaSuccess) {
+    cudaGetLastError();
+    b->flow_mem = nullptr;
+  }
   for (int k = 0; k < kObsSlots && e == cudaSuccess; ++k) {
     b->obs[k].ticket = -1;
     e = cudaEventCreateWithFlags(&b->obs[k].ev, cudaEventDisableTiming);
@@ -628,6 +668,15 @@ int cvf_batch_sweep(cvf_batch* b, const int64_t* sweeps, int32_t n) {
     if (bounds.empty() || bounds.back() != sweeps[act[k]]) bounds.push_back(sweeps[act[k]]);
   if ((int)bounds.size() > kBatchMaxSegments)
     return set_error(CVF_EINVAL, "at most %d distinct step counts per call", kBatchMaxSegments);
+  if (b->tile_cfg < 0) {
+    bool done = false;
+    rc = flow_sweep(b, act, sweeps, any_cmp64(b), &done);
+    if (rc) return rc;
+    if (done) {
+      for (int i : act) b->reps[i].sweep_host += sweeps[i];
+      return CVF_OK;
+    }
+  }
   // the description goes through one of two pinned slots; a slot is
   // rewritten once the copy that read it two calls ago has run
   const int slot = b->work_slot;
@@ -808,6 +857,7 @@ int cvf_batch_destroy(cvf_batch* b) {
     if (o.ev) cudaEventDestroy(o.ev);
   }
   if (b->h_pinned) cudaFreeHost(b->h_pinned);
+  if (b->flow_mem) cudaFree(b->flow_mem);
   if (b->pool) cudaMemPoolDestroy(b->pool);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
   delete b;

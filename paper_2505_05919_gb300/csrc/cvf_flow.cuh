@@ -166,7 +166,7 @@ __device__ __forceinline__ void flow_clerk(PLAN make, FlowSlot* ring, int warps,
 __device__ inline void flow_commit(Ctrl* ctl, const VolumeArgs& vol, cvf_obs* ring,
                                    long long ring_cap, int every, WaveHdr* H, int blocks,
                                    uint32_t* tag, uint32_t end_tag, long long step0,
-                                   long long n_steps) {
+                                   long long n_steps, unsigned int* err) {
   const unsigned int full = 0xFFFFFFFFu;
   const int lane = (int)(threadIdx.x & 31u);
   volatile Ctrl* c = ctl;
@@ -180,7 +180,7 @@ __device__ inline void flow_commit(Ctrl* ctl, const VolumeArgs& vol, cvf_obs* ri
                     ld_acquire(&slot->done) == (unsigned int)blocks;
     const int n = __ffs((int)~__ballot_sync(full, ok)) - 1;
     if (n == 0) {
-      if (flow_idle(idle, H, &ctl->error)) return;
+      if (flow_idle(idle, H, err)) return;
       continue;
     }
     idle = 0;
@@ -264,13 +264,13 @@ __device__ inline void flow_commit(Ctrl* ctl, const VolumeArgs& vol, cvf_obs* ri
 template <typename ARGS>
 __device__ __forceinline__ void flow_books(const ARGS& A, VolumeArgs& V, WaveHdr* H, int blocks,
                                            uint32_t* tag, uint32_t end_tag, long long step0,
-                                           long long n_steps, int every) {
+                                           long long n_steps, int every, unsigned int* err) {
   stage_volume_args(&V, A.vol);
   __syncthreads();
   if (threadIdx.x < 64)
-    wave_engine(A.ctrl, V, A.keys, H, step0, n_steps);
+    wave_engine(A.ctrl, V, A.keys, H, step0, n_steps, err);
   else if (threadIdx.x < 96)
-    flow_commit(A.ctrl, V, A.ring, A.ring_cap, every, H, blocks, tag, end_tag, step0, n_steps);
+    flow_commit(A.ctrl, V, A.ring, A.ring_cap, every, H, blocks, tag, end_tag, step0, n_steps, err);
   if (threadIdx.x >= 96) return;
   // every clerk has reported the last step and looks at the header no more: it is
   // left as the next launch wants it (an abandoned launch leaves it as it is)

@@ -28,6 +28,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
+#include <cstring>
 
 #include "cvf_fastdiv.cuh"
 #include "cvf_flow.cuh"
@@ -45,6 +47,12 @@ constexpr int kFlow2Head = 32;  // words before the copy's cells (word 0: the ta
 struct Flow2Smem {
   Tables2 Tb[2];
   FlowSlot ring[kWaveRing];
+};
+// A block's shared memory: a sweeping block's, or the books' copy of the
+// parameters.
+union Flow2Block {
+  Flow2Smem sweep;
+  VolumeArgs vol;
 };
 
 template <typename SMEM>
@@ -105,28 +113,27 @@ __device__ __forceinline__ CellWords<RNG_WORDS> cell_words(uint32_t c, const Ste
   return w;
 }
 
+// A block of a lattice's launch: the books (b < 0) or block b of `blocks` that
+// sweep.
 template <int RNG_WORDS, bool CMP64, int V, int NT>
-__global__ void __launch_bounds__(NT + 32, 1)
-    k_flow2(const __grid_constant__ LatticeArgs A, const __grid_constant__ Flow2Geom G, WaveHdr* H,
-            uint32_t* copy, long long n_steps, int every) {
-  __shared__ union {
-    Flow2Smem sweep;
-    VolumeArgs vol;  // the engine block's copy of the parameters
-  } U;
+__device__ __forceinline__ void flow2_strips(Flow2Block& U, const LatticeArgs& A,
+                                             const Flow2Geom& G, WaveHdr* H, uint32_t* copy,
+                                             long long n_steps, int every, int b, int blocks,
+                                             unsigned int* err) {
   Ctrl* const ctl = A.ctrl;
-  unsigned int* const err = &ctl->error;
   // the committed step count and the copy's tag: neither changes before every
   // block has taken part in the first (last) step
   const long long step0 = *(volatile long long*)&ctl->sweep;
   const uint32_t tag0 = *(volatile uint32_t*)copy + 1u;
-  if (blockIdx.x == 0) {
-    flow_books(A, U.vol, H, (int)gridDim.x - 1, copy,
-               tag0 + (uint32_t)((unsigned long long)n_steps & 0xFFFFFFu), step0, n_steps, every);
+  if (b < 0) {
+    flow_books(A, U.vol, H, blocks, copy,
+               tag0 + (uint32_t)((unsigned long long)n_steps & 0xFFFFFFu), step0, n_steps, every,
+               err);
     return;
   }
   Flow2Smem& S = U.sweep;
   uint32_t* const F = copy + kFlow2Head;
-  const uint32_t t_lo = (blockIdx.x - 1u) * G.per_block, t_hi = min(t_lo + G.per_block, G.items);
+  const uint32_t t_lo = (uint32_t)b * G.per_block, t_hi = min(t_lo + G.per_block, G.items);
   const int warps = (int)((t_hi - t_lo + 31u) / 32u);
   flow2_setup(S, A, NT + 32);
   __syncthreads();
@@ -253,6 +260,29 @@ __global__ void __launch_bounds__(NT + 32, 1)
   }
 }
 
+template <int RNG_WORDS, bool CMP64, int V, int NT>
+__global__ void __launch_bounds__(NT + 32, 1)
+    k_flow2(const __grid_constant__ LatticeArgs A, const __grid_constant__ Flow2Geom G, WaveHdr* H,
+            uint32_t* copy, long long n_steps, int every) {
+  __shared__ Flow2Block U;
+  flow2_strips<RNG_WORDS, CMP64, V, NT>(U, A, G, H, copy, n_steps, every, (int)blockIdx.x - 1,
+                                        (int)gridDim.x - 1, &A.ctrl->error);
+}
+
+// Many lattices, each with blocks of its own and its own number of steps: the
+// books of all of them first (on SMs apart while there are as many), then the
+// blocks that sweep.
+template <int RNG_WORDS, bool CMP64, int V, int NT>
+__global__ void __launch_bounds__(NT + 32, 1024 / (NT + 32))
+    k_flow2_batch(const __grid_constant__ Flow2Batch B) {
+  __shared__ Flow2Block U;
+  const Flow2Replica& R = B.item[B.of_block[blockIdx.x]];
+  flow2_strips<RNG_WORDS, CMP64, V, NT>(
+      U, R.args, R.geom, R.hdr, R.copy, R.n_steps, 0,
+      blockIdx.x < (unsigned int)B.n ? -1 : (int)(blockIdx.x - R.first_block), (int)R.blocks,
+      B.err);
+}
+
 // ---------------------------------------------------------------------------
 // Small lattices: the same with one word per thread in the shared memory of a
 // thread-block cluster.  A CTA holds a run of words and, on either side, copies
@@ -286,10 +316,7 @@ template <int RNG_WORDS, bool CMP64>
 __global__ void __launch_bounds__(kClusterThreads + 32, 1)
     k_flow2_cluster(const __grid_constant__ LatticeArgs A, const __grid_constant__ Flow2Geom G,
                     WaveHdr* H, long long n_steps, int every) {
-  __shared__ union {
-    Flow2Smem sweep;
-    VolumeArgs vol;
-  } U;
+  __shared__ Flow2Block U;
   __shared__ uint32_t s_word[kClusterThreads + 2 * kClusterHalo];
   __shared__ uint32_t s_no_tag;
   Ctrl* const ctl = A.ctrl;
@@ -402,7 +429,7 @@ __global__ void __launch_bounds__(kClusterThreads + 32, 1)
       reinterpret_cast<uint32_t*>(A.state + (size_t)((step0 + n_steps) & 1) * N)[item] = w;
   };
   if (books)
-    flow_books(A, U.vol, H, (int)gridDim.x - 1, &s_no_tag, 0u, step0, n_steps, every);
+    flow_books(A, U.vol, H, (int)gridDim.x - 1, &s_no_tag, 0u, step0, n_steps, every, err);
   else if (sweeps)
     sweep();
   else if (threadIdx.x >= kClusterThreads)
@@ -422,10 +449,7 @@ template <int RNG_WORDS, bool CMP64, bool ONE, int NT>
 __global__ void __launch_bounds__(NT + 32, 1)
     k_flow2_layer(const __grid_constant__ LatticeArgs A, const __grid_constant__ Flow2Geom G,
                   WaveHdr* H, uint32_t* copy, long long n_steps, int every) {
-  __shared__ union {
-    Flow2Smem sweep;
-    VolumeArgs vol;
-  } U;
+  __shared__ Flow2Block U;
   Ctrl* const ctl = A.ctrl;
   unsigned int* const err = &ctl->error;
   const long long step0 = *(volatile long long*)&ctl->sweep;
@@ -433,7 +457,7 @@ __global__ void __launch_bounds__(NT + 32, 1)
   if (blockIdx.x == 0) {
     flow_books(A, U.vol, H, (int)gridDim.x - 1, copy,
                tag0 + 4u * (uint32_t)((unsigned long long)n_steps & 0xFFFFFFu), step0, n_steps,
-               every);
+               every, err);
     return;
   }
   Flow2Smem& S = U.sweep;
@@ -726,6 +750,110 @@ bool adopt_cluster(Flow2Plan* P, int rng_words, bool cmp64, long long words, lon
 }
 
 }  // namespace
+
+namespace {
+template <int V, int NT>
+const void* batch_kernel(int rng_words, bool cmp64) {
+  if (rng_words == 1)
+    return cmp64 ? (const void*)k_flow2_batch<1, true, V, NT>
+                 : (const void*)k_flow2_batch<1, false, V, NT>;
+  return cmp64 ? (const void*)k_flow2_batch<2, true, V, NT>
+               : (const void*)k_flow2_batch<2, false, V, NT>;
+}
+// Four small blocks per SM for lattices that would leave much of a large one
+// empty, or one large one.
+const Flow2Form kBatchForms[kFlow2BatchForms] = {
+    {1, 224, batch_kernel<1, 224>}, {1, 992, batch_kernel<1, 992>},
+    {2, 224, batch_kernel<2, 224>}, {2, 992, batch_kernel<2, 992>},
+    {4, 224, batch_kernel<4, 224>}, {4, 992, batch_kernel<4, 992>}};
+long long batch_words(int L) {  // of a copy, in whole 128 bytes
+  return ((long long)kFlow2Head + (long long)L * L / 2 + 31) / 32 * 32;
+}
+// The blocks that sweep a lattice, and the items of each.
+void batch_blocks(const Flow2Form& form, int L, Flow2Geom* G, int* blocks) {
+  const long long Lh = L / 2, items = Lh * ((L + form.v - 1) / form.v);
+  const long long n = (items + form.threads - 1) / form.threads;
+  *G = Flow2Geom{};
+  G->items = (uint32_t)items;
+  G->per_block = (uint32_t)(((items + n - 1) / n + 31) / 32 * 32);
+  G->div_row = make_fastdiv((uint32_t)Lh);
+  *blocks = (int)((items + G->per_block - 1) / G->per_block);
+}
+}  // namespace
+
+size_t flow2_batch_scratch() {
+  return (size_t)kFlow2BatchMax * sizeof(WaveHdr) + sizeof(uint32_t) * (size_t)kFlow2BatchWords;
+}
+
+bool flow2_batch_plan(Flow2Batch* B, const int* sides, int n, int rng_words, bool cmp64,
+                      int* slots, int* form) {
+  if (n > kFlow2BatchMax) return false;
+  long long words = 0;
+  for (int i = 0; i < n; ++i) words += batch_words(sides[i]);
+  if (words > kFlow2BatchWords) return false;
+  Flow2Geom G;
+  int own = 0;
+  // The form with the least cost, about its step in 0.01 us beyond 1.2 us: the
+  // chain of a thread's rows, and what the warps of the SM with the most blocks do
+  // (a quarter more where blocks share SMs, and so some of them an SM with a
+  // volume engine, whose FP64 instructions hold back the integer multiplies
+  // beside them).  us per step on 152 SMs, small blocks / large: 64^2 1.8 / 2.3,
+  // 24 of 64^2 2.3 / 2.5, 100 of 64^2 4.8 / do not fit, 24 of 128^2 5.0 / 4.0, 4
+  // of 256^2 3.3 (one row a thread), 4.5 (four) / 3.0, 8 of 256^2 5.3 / 4.4, 12 of
+  // 256^2 7.3 / 8.7, 4 of 512^2 10.2 / 8.5.
+  long long best = LLONG_MAX;
+  for (int f = 0; f < kFlow2BatchForms; ++f) {
+    const Flow2Form& F = kBatchForms[f];
+    if (slots[f] == 0)
+      slots[f] = std::min(kFlow2BatchBlocks,
+                          flow_resident_blocks(F.kernel(rng_words, cmp64), F.threads + 32));
+    long long blocks = n, warps = 0;
+    for (int i = 0; i < n && blocks <= slots[f]; ++i) {
+      batch_blocks(F, sides[i], &G, &own);
+      blocks += own;
+      warps = std::max<long long>(warps, G.per_block / 32);
+    }
+    if (blocks > slots[f]) continue;
+    const long long per_sm = (blocks + sm_count() - 1) / sm_count();
+    const long long cost = 45 * F.v + per_sm * warps * F.v * (per_sm > 1 ? 5 : 4);
+    if (cost < best) {
+      best = cost;
+      *form = f;
+    }
+  }
+  if (best == LLONG_MAX) return false;
+  B->n = n;
+  int next = n;
+  for (int i = 0; i < n; ++i) {
+    batch_blocks(kBatchForms[*form], sides[i], &B->item[i].geom, &own);
+    B->item[i].first_block = (uint32_t)next;
+    B->item[i].blocks = (uint32_t)own;
+    B->of_block[i] = (uint8_t)i;
+    std::memset(B->of_block + next, i, (size_t)own);
+    next += own;
+  }
+  return true;
+}
+
+cudaError_t launch_flow2_batch(Flow2Batch* B, void* scratch, int rng_words, bool cmp64, int form,
+                               cudaStream_t s) {
+  WaveHdr* hdr = reinterpret_cast<WaveHdr*>(scratch);
+  uint32_t* copy = reinterpret_cast<uint32_t*>(hdr + B->n);
+  int blocks = B->n;
+  for (int i = 0; i < B->n; ++i) {
+    B->item[i].hdr = hdr + i;
+    B->item[i].copy = copy;
+    copy += batch_words(B->item[i].args.L);
+    blocks += (int)B->item[i].blocks;
+  }
+  const size_t bytes = (size_t)(reinterpret_cast<char*>(copy) - reinterpret_cast<char*>(scratch));
+  const cudaError_t e = cudaMemsetAsync(scratch, 0, bytes, s);
+  if (e != cudaSuccess) return e;
+  void* args[1] = {B};
+  const Flow2Form& F = kBatchForms[form];
+  return cudaLaunchCooperativeKernel(F.kernel(rng_words, cmp64), dim3(blocks), dim3(F.threads + 32),
+                                     args, 0, s);
+}
 
 Flow2Plan flow2_plan(int L, int schedule, int rng_words, bool cmp64) {
   Flow2Plan P{};

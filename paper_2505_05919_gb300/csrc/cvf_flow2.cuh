@@ -34,6 +34,38 @@ Flow2Plan flow2_plan(int L, int schedule, int rng_words, bool cmp64);
 cudaError_t launch_flow2(const LatticeArgs& A, const Flow2Plan& P, WaveHdr* H, long long n_steps,
                          int every, cudaStream_t s);
 
+// Many lattices in one launch (k_flow2_batch): what the kernel takes by value.
+constexpr int kFlow2BatchBlocks = 640;          // blocks of a launch at most
+constexpr int kFlow2BatchMax = 128;             // lattices of a launch at most
+constexpr long long kFlow2BatchWords = 5 << 17;  // words of its copies at most
+constexpr int kFlow2BatchForms = 6;             // kernels to choose from
+struct Flow2Replica {
+  LatticeArgs args;
+  Flow2Geom geom;
+  WaveHdr* hdr;
+  uint32_t* copy;
+  long long n_steps;             // at most 2^30
+  uint32_t first_block, blocks;  // that sweep
+};
+struct Flow2Batch {
+  int n;
+  unsigned int* err;  // set when a wait gives up or an index check fails
+  uint8_t of_block[kFlow2BatchBlocks];  // the lattice of a block (the first n: the books)
+  Flow2Replica item[kFlow2BatchMax];
+};
+static_assert(sizeof(Flow2Batch) <= 32764, "fits a kernel's parameters");
+
+// Bytes of scratch that any launch fits.
+size_t flow2_batch_scratch();
+// Chooses the form of a launch for n lattices of these sides and its blocks; false
+// if they are not resident at once in any form.  slots[f]: the resident blocks of
+// form f, 0 until asked for.
+bool flow2_batch_plan(Flow2Batch* B, const int* sides, int n, int rng_words, bool cmp64,
+                      int slots[kFlow2BatchForms], int* form);
+// Clears the scratch and launches; args, n_steps and err are the caller's.
+cudaError_t launch_flow2_batch(Flow2Batch* B, void* scratch, int rng_words, bool cmp64, int form,
+                               cudaStream_t s);
+
 // Order of the layered schedule's arms in a step: the Fisher-Yates order drawn
 // from Philox((2^32-2, step, tag 4)), cut before the first arm whose opposite is
 // already in the segment (two or three segments).  Plan word: bits 2i..2i+1 the

@@ -139,7 +139,8 @@ __global__ void __launch_bounds__(kThreads, kWaveBlocksPerSM)
     VolumeArgs* sV = &U.vol;
     stage_volume_args(sV, A.vol);
     __syncthreads();
-    if (threadIdx.x < 64) wave_engine(ctl, *sV, A.keys, H, step0, n_steps);
+    if (threadIdx.x < 64)
+      wave_engine(ctl, *sV, A.keys, H, step0, n_steps, &ctl->error);
     return;
   }
 

@@ -124,7 +124,7 @@ __device__ inline void wave_commit(Ctrl* ctl, const VolumeArgs& vol, cvf_obs* ri
 // volume_decide_pair in the same order, so every move equals the step-by-step
 // chain's.  A proposal that would change the gate ends the walk; it waits for
 // the commit of the step before and is decided with its bonds.  sV is a shared
-// copy of the parameters.
+// copy of the parameters; a wait that gives up sets *err.
 // ---------------------------------------------------------------------------
 constexpr int kWaveTree = 5;  // steps per pass: 31 nodes
 
@@ -152,10 +152,10 @@ __device__ __forceinline__ int lj_shells_near(const VolumeArgs& V, double v, int
 }
 
 __device__ inline void wave_engine(Ctrl* ctl, const VolumeArgs& sV, const RoundKeys& keys,
-                                   WaveHdr* H, long long step0, long long n_steps) {
+                                   WaveHdr* H, long long step0, long long n_steps,
+                                   unsigned int* err) {
   __shared__ WaveTree T;
   const unsigned int full = 0xFFFFFFFFu;
-  unsigned int* const err = &ctl->error;
   const int role = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31u);
   const int n1 = lane + 1;       // 1-based heap index: children 2 n1 (reject), 2 n1 + 1 (accept)
   const int d = 31 - __clz(n1);  // depth (lane 31: below the tree, not used)

@@ -243,3 +243,52 @@ def test_observables_of_many_replicas():
             assert list(got[i]["n_state"]) == [int((arms == v).sum()) for v in range(8)], i
             pairs = sum(int((arms[:, x] == arms[:, y]).sum()) for x in range(4) for y in range(x))
             assert got[i]["n_coop"] == pairs and got[i]["status"] == 0, i
+
+
+# The batched dataflow launch: one, two and four rows a thread in small and large
+# blocks, a lattice of one block and of many, a last warp and a last strip that
+# are partly empty, uneven step counts, the two-word draws, the 64-bit compare,
+# gate flips, the most lattices; a tiled call between two of them.
+FLOW_MIXES = [
+    (1, [(2, {}), (6, dict(q=3)), (34, dict(q=8)), (66, dict(init=oracle.INIT_ORDERED)), (130, {}), (250, {})]),
+    (2, [(2, {}), (30, dict(q=2)), (66, {}), (126, {})]),
+    (1, [(512, {}), (250, dict(q=5)), (66, {}), (4, {})]),
+    (2, [(514, {}), (62, {}), (302, {})]),
+    (1, [(770, {}), (510, {}), (10, {})]),
+    (2, [(766, {}), (530, {})]),
+    (1, [(34, dict(kT=1e-3)), (130, {}), (514, {})]),
+    (1, [(256, {})] * 8),
+    (2, [(128, {})] * 24),
+    (1, [(64, {})] * 100),
+    (1, [(32, {})] * 128),
+    (2, [(16, {})] * 129),
+    (1, [(512, {})] * 4),
+    (1, [(40, dict(gates=True)), (6, dict(gates=True)), (32, {})]),
+]
+
+
+@pytest.mark.parametrize("rng_words,mix", FLOW_MIXES, ids=range(len(FLOW_MIXES)))
+def test_batch_dataflow(rng_words, mix):
+    ps, steps = [], []
+    for i, (L, extra) in enumerate(mix):
+        extra = dict(extra, seed=900 + i, rng_words=rng_words)
+        if extra.pop("gates", False):
+            ps.append(_params(L, 3000.0, 0.1, v_iso_init=1.95, dv_max_frac=0.05, **extra))
+            steps.append(120)
+        elif "kT" in extra:
+            ps.append(params_from_dict(asdict(oracle.OracleParams(L=L, **extra))))
+            steps.append(9)
+        else:
+            ps.append(_params(L, 290.0 + i, 1.0 + i, **extra))
+            steps.append(5 + 7 * (i % 3))
+    with Batch(ps) as b:
+        b.sweep(steps)
+        b.set_tiles(3)
+        b.sweep([3] * len(ps))
+        b.set_tiles(-1)
+        b.sweep([0] + steps[1:])
+        got = [(b.state(i), b.observables(i)) for i in range(len(ps))]
+    for i, p in enumerate(ps):
+        s, o = _solo(p, [steps[i], 3] + ([steps[i]] if i else []))
+        assert np.array_equal(got[i][0], s), i
+        _same(got[i][1], o)
