@@ -204,7 +204,7 @@ int cvf_state_device_ptr(cvf_handle *h, void **dev_ptr);
  * step s + 1 waits only for the tiles around it to finish step s (a
  * wavefront; the volume moves decided ahead by one block; L a multiple of 8
  * and at least 3 x 3 tiles); -1 = automatic (chosen at creation): a lattice
- * small enough (about L <= 1094 on 152 SMs) has no tiles and runs as one
+ * small enough (about L <= 1094 on 152 SMs, 1332 where no tile divides the side) has no tiles and runs as one
  * persistent launch per call in which every word carries its own progress;
  * get_tiles then still names the configuration of the rule for larger ones --
  * the resident form for small lattices, else the largest tile shape whose tiles

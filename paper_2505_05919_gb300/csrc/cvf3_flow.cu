@@ -60,6 +60,11 @@ namespace {
 // blocks of 224, 28.6 with 736).
 constexpr int kFlowThreadsOne = 224, kFlowThreadsMany = 480;
 inline int flow_threads(bool one) { return one ? kFlowThreadsOne : kFlowThreadsMany; }
+// A warp with several groups rests between two looks at its neighbours' words,
+// which take instructions from the warps that sweep (ns; 100^3 22.8 us per step
+// without, 22.1 so; 120^3 35.2 and 34.4; not where rows are no whole groups: 97^3
+// 25.7 and 27.0).
+constexpr unsigned int kRestNs = 300;
 constexpr int kFlowHead = 32;                    // words before the copy's cells (word 0: the tag)
 struct FlowSmem {
   Tables3 Tb[2];  // per gate (the proposals in the first)
@@ -247,6 +252,7 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
           }
           if (__all_sync(full, (int32_t)late >= 0)) break;
           if ((++spins & 255u) == 0u && flow_stop(spins, H, err)) return;
+          if (ALIGNED && !ONE) __nanosleep(kRestNs);
         }
         if (mine && dcheck(cfg < 9u, err, kSiteEta3)) {
           const uint32_t bonds = cube_bonds_packed(v);
@@ -377,6 +383,7 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
             }
             if (__all_sync(full, (int32_t)late >= 0)) break;
             if ((++spins & 255u) == 0u && flow_stop(spins, H, err)) return false;
+            if (ALIGNED && !ONE) __nanosleep(kRestNs);
           }
           if (mine) {
             if (read_eta) {

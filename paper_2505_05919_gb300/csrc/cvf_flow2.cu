@@ -41,6 +41,16 @@
 namespace cvf {
 namespace {
 
+// Up to this many rows a thread the draws of a part are made before its first load
+// (they are the work there is while the neighbours' words come); more of them do
+// not fit the registers (eight rows: 19.3 us per step at 1536^2 with them, 18.3
+// without).
+constexpr int kAheadRows = 4;
+// From this many rows on a warp rests between two looks at its neighbours' words:
+// the looks take instructions from the warps that sweep (ns; 1536^2 18.3 us per
+// step without, 17.7 with 100, 17.0 with 300; 1024^2 7.39 and 7.33).
+constexpr int kRestRows = 4;
+constexpr unsigned int kRestNs = 300;
 constexpr int kFlow2Head = 32;  // words before the copy's cells (word 0: the tag)
 
 // Tables of both gates and the ring of steps.
@@ -120,6 +130,7 @@ __device__ __forceinline__ void flow2_strips(Flow2Block& U, const LatticeArgs& A
                                              const Flow2Geom& G, WaveHdr* H, uint32_t* copy,
                                              long long n_steps, int every, int b, int blocks,
                                              unsigned int* err) {
+  constexpr bool kAhead = V <= kAheadRows;  // the draws of a part are made before its loads
   Ctrl* const ctl = A.ctrl;
   // the committed step count and the copy's tag: neither changes before every
   // block has taken part in the first (last) step
@@ -177,11 +188,14 @@ __device__ __forceinline__ void flow2_strips(Flow2Block& U, const LatticeArgs& A
     int g = 0;
 #pragma unroll
     for (int colour = 0; colour < 2; ++colour) {
-      CellWords<RNG_WORDS> draw[V];
-#pragma unroll
-      for (int k = 0; k < V; ++k) {
+      auto words_of = [&](int k) {
         const uint32_t hi = (odd0 + (uint32_t)(k ^ colour)) & 1u;
-        draw[k] = cell_words<RNG_WORDS>((y0 + k) * L + 2u * p + hi, sd, A.keys);
+        return cell_words<RNG_WORDS>((y0 + k) * L + 2u * p + hi, sd, A.keys);
+      };
+      CellWords<RNG_WORDS> draw[kAhead ? V : 1];
+      if (kAhead) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) draw[kAhead ? k : 0] = words_of(k);
       }
       if (colour == 0) {
         if (!flow_ready(slot, rel, H, err)) return;
@@ -189,28 +203,41 @@ __device__ __forceinline__ void flow2_strips(Flow2Block& U, const LatticeArgs& A
       }
       // what the neighbours' cells (of the other colour) have to show
       const uint32_t need = tag_bits(tag + (uint32_t)colour, tag + (uint32_t)colour);
-      uint32_t side[V], top = 0u, bottom = 0u;
+      // The words beside and above and below the thread's column.  Of two
+      // rows one needs the word to the right, whose low cell is the right
+      // neighbour of its high cell, the other the word to the left, whose high
+      // cell is the left neighbour of its low one; of the words above and below
+      // (rows come in twos) one half each: two halves in a register.
+      constexpr int kPairs = V / 2;
+      uint32_t side[V == 1 ? 1 : kPairs], top = 0u, bottom = 0u;
       for (unsigned int spins = 0;;) {
         uint32_t late = 0u;
+        if (V == 1) {
+          const uint32_t hi = (odd0 + (uint32_t)colour) & 1u;
+          side[0] = ld_flow(F + y0 * Lh + (hi ? right : left));
+          late = (side[0] ^ need) & (hi ? 0x88u : 0x880000u);
+          top = ld_flow(F + up);
+          bottom = ld_flow(F + down);
+          late |= ((top ^ need) | (bottom ^ need)) & (hi ? 0x880000u : 0x88u);
+        } else {
 #pragma unroll
-        for (int k = 0; k < V; ++k) {
-          const uint32_t hi = (odd0 + (uint32_t)(k ^ colour)) & 1u;
-          side[k] = 0u;
-          if ((uint32_t)k < h) {
-            // the low cell's left neighbour is the high cell of the word to the
-            // left, the high cell's right one the low cell to the right
-            side[k] = ld_flow(F + (y0 + k) * Lh + (hi ? right : left));
-            late |= (side[k] ^ need) & (hi ? 0x88u : 0x880000u);
+          for (int m = 0; m < kPairs; ++m) {
+            side[m] = 0u;
+            if ((uint32_t)(2 * m) < h) {
+              const uint32_t xr = ld_flow(F + (y0 + 2 * m + 1 - colour) * Lh + right);
+              const uint32_t xl = ld_flow(F + (y0 + 2 * m + colour) * Lh + left);
+              side[m] = __byte_perm(xr, xl, 0x7610u);
+              late |= (side[m] ^ need) & 0x00880088u;
+            }
           }
+          const uint32_t above = ld_flow(F + up), below = ld_flow(F + down);
+          top = colour ? __byte_perm(below, above, 0x7610u) : __byte_perm(above, below, 0x7610u);
+          bottom = top;
+          late |= (top ^ need) & 0x00880088u;
         }
-        const uint32_t hi0 = (odd0 + (uint32_t)colour) & 1u;          // row 0's half
-        const uint32_t hi1 = (odd0 + h - 1u + (uint32_t)colour) & 1u;  // the last row's
-        top = ld_flow(F + up);
-        bottom = ld_flow(F + down);
-        late |= (top ^ need) & (hi0 ? 0x880000u : 0x88u);
-        late |= (bottom ^ need) & (hi1 ? 0x880000u : 0x88u);
         if (__all_sync(full, late == 0u)) break;
         if ((++spins & 255u) == 0u && flow_stop(spins, H, err)) return;
+        if (V >= kRestRows) __nanosleep(kRestNs);
       }
       if (mine) {
         const Tables2& Tb = S.Tb[g];
@@ -218,14 +245,17 @@ __device__ __forceinline__ void flow2_strips(Flow2Block& U, const LatticeArgs& A
         for (int k = 0; k < V; ++k) {
           if ((uint32_t)k < h) {
             uint32_t acc[4], kk[4];
-            split_draws<RNG_WORDS>(draw[k].u, draw[k].p, q, acc, kk);
+            if (!kAhead) draw[0] = words_of(k);
+            const CellWords<RNG_WORDS>& d = draw[kAhead ? k : 0];
+            split_draws<RNG_WORDS>(d.u, d.p, q, acc, kk);
+            const uint32_t sw = side[k / 2];
             const uint32_t ym = (k == 0) ? top : w[(k > 0) ? k - 1 : 0];
             const uint32_t yp = ((uint32_t)k + 1u == h) ? bottom : w[(k + 1 < V) ? k + 1 : 0];
             const int hi = (V == 1) ? (int)((odd0 + (uint32_t)colour) & 1u) : ((k ^ colour) & 1);
             const uint32_t cell =
-                (V == 1) ? update_cell<CMP64>(w[k], side[k], side[k], ym, yp, hi, acc, kk, q, Tb, pk)
-                : hi ? update_cell<CMP64, 1>(w[k], side[k], side[k], ym, yp, 1, acc, kk, q, Tb, pk)
-                     : update_cell<CMP64, 0>(w[k], side[k], side[k], ym, yp, 0, acc, kk, q, Tb, pk);
+                (V == 1) ? update_cell<CMP64>(w[k], sw, sw, ym, yp, hi, acc, kk, q, Tb, pk)
+                : hi ? update_cell<CMP64, 1>(w[k], sw, sw, ym, yp, 1, acc, kk, q, Tb, pk)
+                     : update_cell<CMP64, 0>(w[k], sw, sw, ym, yp, 0, acc, kk, q, Tb, pk);
             w[k] = put_cell(w[k], cell, hi != 0);
             const uint32_t other = tag + (uint32_t)colour;  // steps the word's other cell has done
             st_flow(F + (y0 + k) * Lh + p,
@@ -679,11 +709,16 @@ bool adopt(Flow2Plan* P, const Flow2Form& form, int rng_words, bool cmp64, long 
 // threads (380), 992 (547): 512^2 2.74 against 2.82 with two rows and 480; two
 // rows, 736 (667): 640^2 3.38 against 3.61 with 992; 992 (774): 768^2 4.49
 // against 5.08 with four and 736; four rows, 736 (943): 896^2 6.0 against 6.35;
-// 992 (1094): 1024^2 7.6 against 11.9 with eight rows and 480, which hides too
-// little latency.
+// 992 (1094): 1024^2 7.4 against 11.9 with eight rows and 480, which hides too
+// little latency.  Eight rows and 736 threads (1332) where the wavefront's tiles
+// do not divide the side: 1096^2 10.3 against 12.9 with the wavefront, 1200^2 11.0
+// / 14.6, 1300^2 14.0 / 21.5, but 1152^2 12.4 / 12.3 and 1280^2 14.1 / 13.5; with
+// two-word draws where rows are not 16-byte aligned, too: 1300^2 19.9 / 25.2, but
+// 1120^2 16.6 / 15.4.
 const Flow2Form kStrips[] = {{1, 480, flow2_kernel<1, 480>}, {1, 992, flow2_kernel<1, 992>},
                              {2, 736, flow2_kernel<2, 736>}, {2, 992, flow2_kernel<2, 992>},
-                             {4, 736, flow2_kernel<4, 736>}, {4, 992, flow2_kernel<4, 992>}};
+                             {4, 736, flow2_kernel<4, 736>}, {4, 992, flow2_kernel<4, 992>},
+                            {8, 736, flow2_kernel<8, 736>}};
 // The layered sweep: one group a thread (512^2 4.3 us per step), or several with
 // as many warps as fit (1024^2 14.6 us with 992 threads, 16.4 with 736, 17.3
 // with 480; 4096^2 195, 201, 240).
@@ -761,7 +796,9 @@ const void* batch_kernel(int rng_words, bool cmp64) {
                : (const void*)k_flow2_batch<2, false, V, NT>;
 }
 // Four small blocks per SM for lattices that would leave much of a large one
-// empty, or one large one.
+// empty, or one large one.  (Eight rows would take batches of up to twice the
+// cells, but are no faster than the tiled sweep there: 5 of 512^2 18.1 us per step
+// against 15.3, 24 of 256^2 16.4 / 16.8, 8 of 512^2 17.7 / 20.3.)
 const Flow2Form kBatchForms[kFlow2BatchForms] = {
     {1, 224, batch_kernel<1, 224>}, {1, 992, batch_kernel<1, 992>},
     {2, 224, batch_kernel<2, 224>}, {2, 992, batch_kernel<2, 992>},
@@ -871,7 +908,8 @@ Flow2Plan flow2_plan(int L, int schedule, int rng_words, bool cmp64) {
   if (adopt_cluster(&P, rng_words, cmp64, Lh * L, Lh)) return P;
   P.copy_words = (size_t)kFlow2Head + (size_t)(Lh * L);
   for (const Flow2Form& form : kStrips)
-    if (adopt(&P, form, rng_words, cmp64, Lh * ((L + form.v - 1) / form.v), true)) break;
+    if ((form.v < 8 || L % (rng_words == 1 ? 128 : 8) != 0) &&
+        adopt(&P, form, rng_words, cmp64, Lh * ((L + form.v - 1) / form.v), true)) break;
   return P;
 }
 

@@ -635,6 +635,8 @@ DATAFLOW = [
     (778, 3, 1, 0, dict(q=5, rng_words=2)),
     (946, 3, 1, 0, {}),
     (1094, 3, 3, 0, dict(kT=1e-3)),
+    (1096, 2, 1, 0, {}),
+    (1322, 2, 1, 0, dict(rng_words=2)),
     (6, 400, 1, 0, dict(gates=True)),
     (70, 200, 1, 0, dict(gates=True)),
     (2, 80, 1, 1, {}),
