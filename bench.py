@@ -88,7 +88,7 @@ COUNTERS_FILE = os.path.join(ROOT, "profiles", "k_sweep_wave_L4096_counters.json
 SWEEP_SOURCES = ("paper_2505_05919_gb300/csrc/cvf_tile.cuh", "paper_2505_05919_gb300/csrc/cvf_lattice.cu",
                  "paper_2505_05919_gb300/csrc/cvf_lattice.cuh", "paper_2505_05919_gb300/csrc/cvf_device.cuh",
                  "paper_2505_05919_gb300/csrc/cvf_tma.cuh", "paper_2505_05919_gb300/csrc/cvf_wave.cu",
-                 "paper_2505_05919_gb300/csrc/cvf_fastdiv.cuh")
+                 "paper_2505_05919_gb300/csrc/cvf_wave.cuh", "paper_2505_05919_gb300/csrc/cvf_fastdiv.cuh")
 
 
 def sweep_source_hash() -> str:

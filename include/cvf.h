@@ -204,8 +204,9 @@ int cvf_state_device_ptr(cvf_handle *h, void **dev_ptr);
  * step s + 1 waits only for the tiles around it to finish step s (a
  * wavefront; the volume moves decided ahead by one block; L a multiple of 8
  * and at least 3 x 3 tiles); -1 = automatic (chosen at creation): a lattice
- * small enough (about L <= 1094 on 152 SMs, 1332 where no tile divides the side) has no tiles and runs as one
- * persistent launch per call in which every word carries its own progress;
+ * small enough (about L <= 1094 on 152 SMs, 1332 where no tile divides the
+ * side) has no tiles and runs as one persistent launch per call in which every
+ * word carries its own progress;
  * get_tiles then still names the configuration of the rule for larger ones --
  * the resident form for small lattices, else the largest tile shape whose tiles
  * fill every resident block, swept as a wavefront from L = 256 up -- and the
@@ -338,8 +339,11 @@ int cvf_batch_get_state(cvf_batch *b, int32_t replica, uint16_t *host,
  * over the replicas the call advances is at least the kernel's co-resident
  * blocks; else the smallest tile, with 512-thread blocks (config 11) when
  * its count is below a quarter of the blocks and 256-thread blocks (config
- * 3) otherwise.  cvf_batch_get_tiles returns the setting and the
- * configuration the last call used (-1 before any call). */
+ * 3) otherwise.  A call whose replicas are resident at once (up to about 1.2
+ * million cells in at most 128 replicas on 152 SMs) then runs without tiles, as
+ * one launch in which every word carries its own progress; set a configuration
+ * to run its tiles.  cvf_batch_get_tiles returns the setting and the
+ * configuration that the last call's rule chose (-1 before any call). */
 int cvf_batch_set_tiles(cvf_batch *b, int32_t config);
 int cvf_batch_get_tiles(cvf_batch *b, int32_t *config, int32_t *last_used);
 int cvf_batch_tile_config(int32_t config, int32_t *rows, int32_t *words);

@@ -70,7 +70,8 @@ class Batch:
         default) to let each call choose the largest 256-thread tile that
         still gives every co-resident block a tile (the smallest tile, with
         512-thread blocks when its tiles are under a quarter of the
-        blocks)."""
+        blocks), or to run without tiles where all replicas are resident at
+        once (about 1.2 million cells)."""
         _capi.cvf_batch_set_tiles(self.b, config)
 
     def tiles(self) -> tuple:
