@@ -23,7 +23,7 @@
 // (0.27 to 0.5 us between SMs), the four arm updates -- up to about 512^2, the
 // instructions of the cells beyond (the launches and waits that it replaces
 // took 2.7 us per step at 64^2, 8.2 at 258^2, 7.3 at 512^2 and 11.9 at 1024^2;
-// now 1.3, 1.9, 2.7 and 7.6).  The draws of a part are made before its first
+// now 1.3, 1.9, 2.7 and 7.4).  The draws of a part are made before its first
 // load.
 #include <cuda_runtime.h>
 
@@ -42,9 +42,9 @@ namespace cvf {
 namespace {
 
 // Up to this many rows a thread the draws of a part are made before its first load
-// (they are the work there is while the neighbours' words come); more of them do
-// not fit the registers (eight rows: 19.3 us per step at 1536^2 with them, 18.3
-// without).
+// (they are the work there is while the neighbours' words come: 900^2 6.0 us per
+// step, 6.3 without; 1024^2 7.5 and 7.7); the draws of more rows do not fit the
+// registers.
 constexpr int kAheadRows = 4;
 // From this many rows on a warp rests between two looks at its neighbours' words:
 // the looks take instructions from the warps that sweep (ns; 1536^2 18.3 us per
@@ -720,7 +720,7 @@ const Flow2Form kStrips[] = {{1, 480, flow2_kernel<1, 480>}, {1, 992, flow2_kern
                              {4, 736, flow2_kernel<4, 736>}, {4, 992, flow2_kernel<4, 992>},
                             {8, 736, flow2_kernel<8, 736>}};
 // The layered sweep: one group a thread (512^2 4.3 us per step), or several with
-// as many warps as fit (1024^2 14.6 us with 992 threads, 16.4 with 736, 17.3
+// as many warps as fit (1024^2 14.0 us with 992 threads, 16.4 with 736, 17.3
 // with 480; 4096^2 195, 201, 240).
 const Flow2Form kLayerOne = {0, 480, flow2_layer_kernel<true, 480>};
 const Flow2Form kLayerMany = {0, 992, flow2_layer_kernel<false, 992>};

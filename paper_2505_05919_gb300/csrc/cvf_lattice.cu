@@ -841,9 +841,9 @@ int wave_scratch(cvf_handle* h, int shape) {
 }
 
 // The automatic configuration of the lattices that the dataflow sweep does not
-// take (Flow2Plan; it is faster wherever it fits: 64^2 1.8 against 2.7 us per
-// step with the resident form, 258^2 1.9 / 7.9 tiled, 512^2 2.7 / 7.0 and 1024^2
-// 7.6 / 11.2 with the wavefront): the resident form for small lattices; the
+// take (Flow2Plan; it is faster wherever it fits: 64^2 1.3 against 2.7 us per
+// step with the resident form, 258^2 2.0 / 7.9 tiled, 512^2 2.7 / 7.0 and 1024^2
+// 7.4 / 11.2 with the wavefront): the resident form for small lattices; the
 // wavefront sweep from 256^2 up, with the tiled sweep's shape rule (the
 // largest shape with at least as many tiles as the tiled sweep has resident
 // blocks: the fastest wavefront shape at 768^2, 1536^2, 2048^2 and from
@@ -859,8 +859,8 @@ int wave_scratch(cvf_handle* h, int shape) {
 // wavefront stays ahead).
 constexpr int kWaveAutoMin = 256;
 // The layered schedule runs as a dataflow sweep (cvf_flow2.cu) up to this side:
-// it is faster than a launch per segment at every side measured (1024^2 14.6
-// against 31.8 us per step, 2048^2 55.5 / 80.2, 4096^2 195 / 260), but its copy
+// it is faster than a launch per segment at every side measured (1024^2 14.0
+// against 31.8 us per step, 2048^2 54.1 / 80.2, 4096^2 195 / 260), but its copy
 // doubles the lattice's memory (4 bytes a cell).
 constexpr int kFlowLayerMaxSide = 16384;
 int auto_config(const cvf_handle* h) {
