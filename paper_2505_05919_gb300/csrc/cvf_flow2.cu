@@ -718,7 +718,7 @@ bool adopt(Flow2Plan* P, const Flow2Form& form, int rng_words, bool cmp64, long 
 const Flow2Form kStrips[] = {{1, 480, flow2_kernel<1, 480>}, {1, 992, flow2_kernel<1, 992>},
                              {2, 736, flow2_kernel<2, 736>}, {2, 992, flow2_kernel<2, 992>},
                              {4, 736, flow2_kernel<4, 736>}, {4, 992, flow2_kernel<4, 992>},
-                            {8, 736, flow2_kernel<8, 736>}};
+                             {8, 736, flow2_kernel<8, 736>}};
 // The layered sweep: one group a thread (512^2 4.3 us per step), or several with
 // as many warps as fit (1024^2 14.0 us with 992 threads, 16.4 with 736, 17.3
 // with 480; 4096^2 195, 201, 240).
