@@ -66,7 +66,9 @@ constexpr uint32_t kFlowMaxGroupsRagged = 112u * 112u * 112u / 4u;
 // 16-byte vectors.  Otherwise every cell computes its own coordinates.
 // Launch 0 has one extra block (block 0) that decides the next step's volume
 // move early when it cannot depend on the bonds (no gate change); launch
-// kLaunches3 - 1 commits the step.
+// kLaunches3 - 1 commits the step.  The plan is made from ctl->sweep in launch 0
+// only: a last launch without a segment commits as soon as its block 0 runs, and
+// a block that starts after that must still find the committed step's plan.
 // ---------------------------------------------------------------------------
 template <bool ALIGNED, bool CMP64>
 __global__ void __launch_bounds__(kThreads3, 4) k_pass3(Args3 A, int launch) {
@@ -77,9 +79,16 @@ __global__ void __launch_bounds__(kThreads3, 4) k_pass3(Args3 A, int launch) {
   Ctrl* ctl = A.ctrl;
   const bool fin = (launch == kLaunches3 - 1);
   if (threadIdx.x == 0) {
-    const unsigned long long plan = make_plan(ctl->sweep, A.keys);
+    unsigned long long plan;
+    if (launch == 0) {
+      plan = make_plan(ctl->sweep, A.keys);
+      if (blockIdx.x == 0) ctl->plan = plan;
+    } else {
+      plan = ctl->plan;
+    }
     s_seg = launch < plan_segments(plan) ? plan_segment(plan, launch) : 0u;
-    // N_q' is accumulated by the launch that finishes a recorded step
+    // N_q' is accumulated by the launch that finishes a recorded step (which
+    // every block of it takes part in: the step is not committed before)
     s_rec = (launch == plan_segments(plan) - 1 &&
              step_recorded(ctl->record_every, ctl->sweep)) ? 1 : 0;
   }

@@ -332,7 +332,10 @@ struct Ctrl {
   int ahead_g;
   int ahead_acc;
   int ahead_state;
-  int plan;             // cubic lattice: launch plan of the current step's six passes
+  int pad0;
+  // arm order of the current step, where a step is several launches: written by
+  // the first of them and read by the others
+  unsigned long long plan;
   // per-step accumulators (zero between steps)
   unsigned long long acc_hb;
   unsigned long long acc_pairs;

@@ -377,3 +377,40 @@ def test_lattice3_dataflow_sweep(L, eta, steps, every, extra):
     assert recount == (o["n_hb_raw"], o["n_coop"])
     for i, (g, w) in enumerate(zip(got, want)):
         _same(g, w, ("record", i))
+
+
+@pytest.mark.parametrize("L,steps,eta", [(130, 640, 1), (115, 320, 0), (132, 320, 1)])
+def test_lattice3_launch_sweep_beside_another_cube(L, steps, eta):
+    """Cubes above the dataflow sweep's sides run as launches whose blocks, with
+    another cube's kernels on the GPU, do not all start together: a block of a
+    step's last launch that starts after the step is committed must still go by
+    that step's plan.  Each of two cubes on streams of their own equals the same
+    cube run alone."""
+    import torch
+    ps = [params_from_dict(asdict(oracle.physical_params3(300.0, 0.1, L=L, seed=s, eta_moves=eta)))
+          for s in (61, 62)]
+    alone = []
+    for p in ps:
+        with Lattice3(p) as lat:
+            lat.sweep(steps, 16)
+            alone.append((lat.state(), lat.eta(), lat.observables(), lat.drain()[0]))
+    streams = [torch.cuda.Stream() for _ in ps]
+    torch.cuda.synchronize()
+    lats = [Lattice3(p, stream=s) for p, s in zip(ps, streams)]
+    try:
+        for _ in range(steps // 64):
+            for lat in lats:
+                lat.sweep(64, 16)
+        for lat, (s, e, o, series) in zip(lats, alone):
+            assert np.array_equal(lat.state(), s)
+            assert np.array_equal(lat.eta(), e)
+            got = lat.observables()
+            _same(got, o, L)
+            assert lat.recount() == (got["n_hb_raw"], got["n_coop"])
+            records, _ = lat.drain()
+            assert len(records) == len(series) == steps // 16
+            for g, w in zip(records, series):
+                _same(g, w, L)
+    finally:
+        for lat in lats:
+            lat.close()
