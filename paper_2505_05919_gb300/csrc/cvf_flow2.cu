@@ -87,16 +87,26 @@ __device__ __forceinline__ bool flow_ready(const FlowSlot& slot, long long rel, 
 }
 
 // A warp's counts of a step (and N_q' in the 16-bit lanes v, v + 4 of h[v])
-// into its slot.
+// into its slot.  MANY: the warp may have counted more than the 65535 arms of one
+// state that the lanes of its sum hold, so the two are summed apart.
+template <bool MANY = false>
 __device__ __forceinline__ void flow_report2(FlowSlot& slot, const TileCounts& cnt, bool rec,
                                              const uint32_t h[4]) {
   if (rec) {
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      const uint32_t lanes = __reduce_add_sync(0xFFFFFFFFu, h[v]);
+      uint32_t low, high;
+      if (MANY) {
+        low = __reduce_add_sync(0xFFFFFFFFu, h[v] & 0xFFFFu);
+        high = __reduce_add_sync(0xFFFFFFFFu, h[v] >> 16);
+      } else {
+        const uint32_t lanes = __reduce_add_sync(0xFFFFFFFFu, h[v]);
+        low = lanes & 0xFFFFu;
+        high = lanes >> 16;
+      }
       if ((threadIdx.x & 31u) == 0u) {
-        if (lanes & 0xFFFFu) atomicAdd(&slot.hist[v], lanes & 0xFFFFu);
-        if (lanes >> 16) atomicAdd(&slot.hist[v + 4], lanes >> 16);
+        if (low) atomicAdd(&slot.hist[v], low);
+        if (high) atomicAdd(&slot.hist[v + 4], high);
       }
     }
   }
@@ -559,6 +569,8 @@ __global__ void __launch_bounds__(NT + 32, 1)
     const bool rec = step_recorded(every, step);
     const int nseg = 1 + __popc(plan >> 9);
     TileCounts cnt{0, 0, 0};
+    // a group adds up to 16 arms of one state to a thread's 16-bit lane, which holds
+    // kFlow2LayerGroups of them (449 at kFlowLayerMaxSide on 152 SMs)
     uint32_t hist[4] = {0u, 0u, 0u, 0u};
     for (int j = 0; j < nseg; ++j) {
       const uint32_t arms = layer_segment(plan, j);
@@ -661,7 +673,7 @@ __global__ void __launch_bounds__(NT + 32, 1)
         __syncwarp();
       }
     }
-    flow_report2(slot, cnt, rec, hist);
+    flow_report2<!ONE>(slot, cnt, rec, hist);
   }
 }
 
@@ -724,6 +736,8 @@ const Flow2Form kStrips[] = {{1, 480, flow2_kernel<1, 480>}, {1, 992, flow2_kern
 // with 480; 4096^2 195, 201, 240).
 const Flow2Form kLayerOne = {0, 480, flow2_layer_kernel<true, 480>};
 const Flow2Form kLayerMany = {0, 992, flow2_layer_kernel<false, 992>};
+// Groups of a thread at most: their arms of one state fit its 16-bit counters.
+constexpr uint32_t kFlow2LayerGroups = 65535u / 16u;
 // The cluster form: at most fifteen CTAs with words (128^2) and one with the
 // books; a CTA for every so many words (64^2 1.27 us per step with 64 or 128,
 // 1.30 with 256, 1.56 with 544).
@@ -899,8 +913,10 @@ Flow2Plan flow2_plan(int L, int schedule, int rng_words, bool cmp64) {
     P.geom.groups_x = (uint32_t)gx;
     P.geom.div_row = make_fastdiv((uint32_t)gx);
     P.copy_words = (size_t)kFlow2Head + 4 * (size_t)groups;
-    if (!adopt(&P, kLayerOne, rng_words, cmp64, groups, true))
-      adopt(&P, kLayerMany, rng_words, cmp64, groups, false);
+    if (!adopt(&P, kLayerOne, rng_words, cmp64, groups, true) &&
+        adopt(&P, kLayerMany, rng_words, cmp64, groups, false) &&
+        P.geom.per_block > (uint32_t)kLayerMany.threads * kFlow2LayerGroups)
+      P.blocks = 0;  // (a GPU of few SMs)
     return P;
   }
   const long long Lh = L / 2;

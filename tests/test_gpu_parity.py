@@ -672,3 +672,21 @@ def test_dataflow_sweep(L, K, every, layered, extra):
     assert counts == (o["n_hb_raw"], o["n_coop"])
     for i, (a, b) in enumerate(zip(got, want)):
         assert_obs_equal(a, b, ("record", i))
+
+
+@pytest.mark.parametrize("L,q,init,kT", [(10000, 6, oracle.INIT_ORDERED, 1e-3), (16384, 6, oracle.INIT_ORDERED, 1e-3),
+                                         (16384, 2, oracle.INIT_RANDOM, 5.0)])
+def test_layered_series_counts_of_large_lattices(L, q, init, kT):
+    """N_q' recorded by the layered sweep where a warp sees more than 65535 arms
+    of one state in a step (128 groups a thread and more): it equals the count of
+    the lattice itself and adds up to 4 N."""
+    op = oracle.OracleParams(L=L, q=q, init=init, kT=kT, seed=L + q, schedule=oracle.SCHED_LAYERED)
+    with Lattice(params_from_dict(asdict(op))) as lat:
+        lat.sweep(1, 1)
+        o = lat.observables()
+        records, _ = lat.drain()
+        assert lat.recount() == (o["n_hb_raw"], o["n_coop"])
+    assert len(records) == 1 and sum(o["n_state"]) == 4 * L * L
+    assert list(records[0]["n_state"]) == list(o["n_state"])
+    assert max(o["n_state"]) > 4 * L * L // 4
+    assert_obs_equal(records[0], o)
