@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(kObserveThreads)
 
 cudaError_t launch_observe(const ObserveArgs& A, int items, long long most, bool cubic,
                            cudaStream_t s) {
-  const dim3 grid((unsigned)observe_blocks(most, sm_count()), (unsigned)items);
+  const dim3 grid((unsigned)observe_blocks(most, sm_count(), cubic ? 6 : 4), (unsigned)items);
   if (cubic)
     k_observe<true><<<grid, kObserveThreads, 0, s>>>(A);
   else

@@ -30,12 +30,16 @@ struct ObserveArgs {
 };
 
 constexpr int kObserveThreads = 256;
-// Blocks per lattice: two 8- or 16-byte loads a thread for small ones, and never
-// more than 2^12 of them in one thread's 16-bit lanes (L <= 65534: 1216 blocks).
-inline int observe_blocks(long long N, int sms) {
+// Blocks per lattice of N cells of `arms` arms: two loads of four cells a thread
+// for small ones, eight blocks an SM for large ones, but as many as it takes for
+// a thread's arms of one state to fit its 16-bit lanes.
+inline int observe_blocks(long long N, int sms, int arms) {
   const long long want = (N + 8 * kObserveThreads - 1) / (8 * kObserveThreads);
   const long long most = 8ll * sms;
-  return (int)(want < 1 ? 1 : want > most ? most : want);
+  const long long loads = 65535 / (4 * arms);  // of a thread at most
+  const long long least = (N + 4 * kObserveThreads * loads - 1) / (4 * kObserveThreads * loads);
+  const long long blocks = want > most ? most : want;
+  return (int)(blocks > least ? blocks : least);
 }
 
 // Enqueues the observation of items (at most kObserveItems) of lattices of up
