@@ -409,8 +409,9 @@ int launch_error(unsigned int err) {
 }
 
 // (Re)allocates a ticket slot's staging for cap records; the slot's last
-// copy must be done.
-cudaError_t grow_obs_slot(cvf_batch::ObsSlot& o, int cap) {
+// copy must be done.  The counters are cleared on the batch's stream, which the
+// launches that count into them follow (it may not wait for the default one).
+cudaError_t grow_obs_slot(cvf_batch::ObsSlot& o, int cap, cudaStream_t s) {
   if (o.d_counts) cudaFree(o.d_counts);
   if (o.h_obs) cudaFreeHost(o.h_obs);
   o.d_counts = nullptr;
@@ -418,7 +419,7 @@ cudaError_t grow_obs_slot(cvf_batch::ObsSlot& o, int cap) {
   o.cap = 0;
   const size_t bytes = sizeof(unsigned long long) * 10 * cap;
   cudaError_t e = cudaMalloc(&o.d_counts, bytes);
-  if (e == cudaSuccess) e = cudaMemset(o.d_counts, 0, bytes);
+  if (e == cudaSuccess) e = cudaMemsetAsync(o.d_counts, 0, bytes, s);
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&o.h_obs), sizeof(cvf_obs) * cap);
   if (e == cudaSuccess) o.cap = cap;
   return e;
@@ -473,7 +474,7 @@ int cvf_batch_create(const cvf_params* params, int32_t n, void* stream, cvf_batc
     b->obs[k].ticket = -1;
     e = cudaEventCreateWithFlags(&b->obs[k].ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&b->obs[k].h_err), 64);
-    if (e == cudaSuccess) e = grow_obs_slot(b->obs[k], 16);
+    if (e == cudaSuccess) e = grow_obs_slot(b->obs[k], 16, b->stream);
   }
   for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
     e = cudaEventCreateWithFlags(&b->ev_work[k], cudaEventDisableTiming);
@@ -736,7 +737,7 @@ int cvf_batch_observables_enqueue(cvf_batch* b, const int32_t* replicas, int32_t
   if (n > o.cap) {
     int cap = o.cap;
     while (cap < n) cap *= 2;
-    CVF_CUDA_CHECK(grow_obs_slot(o, cap));
+    CVF_CUDA_CHECK(grow_obs_slot(o, cap, b->stream));
   }
   // the records (and, with the first, the last launch's error word) go to the
   // pinned slot from the kernel; kObserveItems replicas per launch

@@ -292,3 +292,23 @@ def test_batch_dataflow(rng_words, mix):
         s, o = _solo(p, [steps[i], 3] + ([steps[i]] if i else []))
         assert np.array_equal(got[i][0], s), i
         _same(got[i][1], o)
+
+
+def test_observables_counters_follow_the_batch_stream():
+    """A slot that grows for more records clears its new counters in the order
+    of the batch's stream, whatever the default stream is doing."""
+    import torch
+    s = torch.cuda.Stream()
+    for n in (40, 80, 160):
+        with Batch([_params(16, seed=500 + i) for i in range(n)], stream=s) as b:
+            b.sweep([2] * n)
+            b.sync()
+            torch.cuda._sleep(100_000_000)       # the default stream is busy meanwhile
+            got = b.observables_many(list(range(n)))
+            again = b.observables_many(list(range(n)))
+            torch.cuda.synchronize()
+            for i in range(0, n, 7):
+                w = b.state(i).reshape(-1).astype(np.int64)
+                arms = np.stack([(w >> (4 * a)) & 7 for a in range(4)])
+                assert list(got[i]["n_state"]) == [int((arms == v).sum()) for v in range(8)], i
+                _same(got[i], again[i])
