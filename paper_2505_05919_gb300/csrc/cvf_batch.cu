@@ -104,6 +104,7 @@ struct cvf_batch {
   cudaMemPool_t pool;
   std::vector<Replica> reps;
   int rng_words;       // shared by all replicas (-1 while empty)
+  int kernel_words;    // the one whose kernels graph, grid and flow_slots are of
   int tile_cfg;        // -1: chosen per call
   int last_cfg;        // the shape the last call used
   ReplicaDesc* d_reps;
@@ -172,7 +173,8 @@ void free_replica(Replica& r, cudaStream_t s) {
   r = Replica();
 }
 
-// Captured graphs hold device addresses; drop them when a buffer moves.
+// Captured graphs hold device addresses and kernels; drop them when a buffer
+// moves or the kernels change.
 void drop_graphs(cvf_batch* b) {
   for (int c = 0; c < kNumTileConfigs; ++c)
     for (int k = 0; k < 2; ++k) {
@@ -451,6 +453,7 @@ int cvf_batch_create(const cvf_params* params, int32_t n, void* stream, cvf_batc
   if (!b) return set_error(CVF_ENOMEM, "host allocation failed");
   b->stream = reinterpret_cast<cudaStream_t>(stream);
   b->rng_words = -1;
+  b->kernel_words = -1;
   b->tile_cfg = -1;
   b->last_cfg = -1;
   cudaError_t e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
@@ -570,6 +573,12 @@ int cvf_batch_add(cvf_batch* b, const cvf_params* p, int32_t* replica) {
     b->reps[id] = r;
   }
   if (b->rng_words < 0) b->rng_words = p->rng_words;
+  if (b->kernel_words != b->rng_words) {
+    drop_graphs(b);
+    std::memset(b->grid, 0, sizeof(b->grid));
+    std::memset(b->flow_slots, 0, sizeof(b->flow_slots));
+    b->kernel_words = b->rng_words;
+  }
   b->reps_dirty = true;
   *replica = id;
   return CVF_OK;

@@ -312,3 +312,25 @@ def test_observables_counters_follow_the_batch_stream():
                 arms = np.stack([(w >> (4 * a)) & 7 for a in range(4)])
                 assert list(got[i]["n_state"]) == [int((arms == v).sum()) for v in range(8)], i
                 _same(got[i], again[i])
+
+
+@pytest.mark.parametrize("first,then", [(1, 2), (2, 1)])
+@pytest.mark.parametrize("cfg", [-1, 0, 3, 11])
+def test_batch_emptied_and_refilled_with_other_draws(first, then, cfg):
+    """A batch that lost its last replica takes replicas of the other
+    rng_words, and sweeps them with that number of draws."""
+    sides = [64, 130, 258, 34]
+    with Batch([_params(L, seed=70 + L, rng_words=first) for L in sides]) as b:
+        b.set_tiles(cfg)
+        b.sweep([6] * 4)
+        for i in range(4):
+            b.remove(i)
+        ps = [_params(L, seed=80 + L, rng_words=then) for L in sides]
+        ids = [b.add(p) for p in ps]
+        assert sorted(ids) == [0, 1, 2, 3]
+        b.sweep([6] * 4)
+        got = [(b.state(i), b.observables(i)) for i in ids]
+    for (s, o), p in zip(got, ps):
+        want, ow = _solo(p, [6])
+        assert np.array_equal(s, want), (p.L, cfg)
+        _same(o, ow)
