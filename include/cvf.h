@@ -476,12 +476,13 @@ int cvf3_state_device_ptr(cvf3_handle *h, void **dev_ptr);
  * 16 <= L <= 64; 16 CTAs where L is a multiple of 16 from 32 up and the GPU
  * can place such a cluster, else 8; the z-planes split among the CTAs; with
  * eta moves each CTA moves the cubes whose lower plane it holds), 0 runs the
- * cube from global memory, -1 chooses.  The results do not depend on the form;
- * the call waits for the stream.  CVF_EINVAL for mode 1 where it does not
- * apply.  From global memory -- and by the automatic choice (-1, the default
- * at creation) -- a cube up to 128^3 runs as one persistent launch per call,
- * in which every word carries its own progress and stays in the registers of
- * the thread that owns it up to 51^3; a larger one as four launches per step.
+ * step as launches over the cube in global memory (four per step, five with eta
+ * moves), -1 chooses.  The results do not depend on the form; the call waits
+ * for the stream.  CVF_EINVAL for mode 1 where it does not apply.  The
+ * automatic choice (-1, the default at creation) runs a cube up to 128^3 (up to
+ * 112^3 without eta moves where L is no multiple of 4) as one persistent launch
+ * per call, in which every word carries its own progress and stays in the
+ * registers of the thread that owns it up to 51^3, and a larger one as launches.
  * cvf3_get_resident: 1 after mode 1, and under the automatic choice for the
  * small cubes that mode 1 takes (up to 24, and 32 with a 16-CTA cluster). */
 int cvf3_set_resident(cvf3_handle *h, int32_t mode);

@@ -979,7 +979,8 @@ struct cvf3_handle {
   bool resident;  // the small-cube form (reported by cvf3_get_resident)
   bool cluster;   // asked for: one cluster's shared memory holds the cube during a call
   int res_ctas;   // CTAs of that cluster (0 until it is first needed)
-  bool flow;        // the dataflow sweep, where no cluster was asked for
+  bool flow;        // the dataflow sweep takes the cube
+  bool use_flow;    // ... and neither the cluster nor the launches were asked for
   Flow3Plan plan;
   WaveHdr* wave;    // its scratch and, behind it, its tagged copy of the cube
   int grid;
@@ -1201,6 +1202,7 @@ int cvf3_create(const cvf_params* p, void* stream, void* dev_state, cvf3_handle*
     }
   }
   h->cluster = h->resident && !h->flow;
+  h->use_flow = h->flow;
   h->grid_count = (int)std::max<long long>(
       1, std::min<long long>((h->N + kThreads3 - 1) / kThreads3, (long long)sm_count() * 8));
   h->grid_eta = (int)std::max<long long>(
@@ -1236,7 +1238,7 @@ int cvf3_sweep(cvf3_handle* h, int64_t n_sweeps, int32_t record_every) {
     return set_error(CVF_EINVAL, "n_sweeps=%lld, record_every=%d must be >= 0",
                      (long long)n_sweeps, record_every);
   if (n_sweeps == 0) return CVF_OK;
-  if (h->cluster || h->flow) {
+  if (h->cluster || h->use_flow) {
     if (h->cluster && !h->res_ctas) h->res_ctas = resident3_ctas(h->args, h->cmp64);
     // the kernels' step counters are 32-bit
     const long long chunk = h->cluster ? 1ll << 16 : 1ll << 30;
@@ -1434,6 +1436,7 @@ int cvf3_set_resident(cvf3_handle* h, int32_t mode) {
   CVF_CUDA_CHECK(cudaStreamSynchronize(h->stream));
   h->resident = (mode == 1) || (mode == -1 && resident3_auto(h->args, h->cmp64));
   h->cluster = h->resident && (mode == 1 || !h->flow);
+  h->use_flow = h->flow && mode == -1;
   return CVF_OK;
 }
 

@@ -86,8 +86,8 @@ class Lattice3:
 
     def set_resident(self, mode: int) -> None:
         """1: the cube resident in one thread-block cluster during each call
-        (L a multiple of 8, 16 <= L <= 64); 0: from global memory; -1: choose
-        (cvf3_set_resident in cvf.h)."""
+        (L a multiple of 8, 16 <= L <= 64); 0: launches for every step; -1:
+        choose (one persistent launch per call up to about 128^3)."""
         _capi.cvf3_set_resident(self.h, mode)
 
     def resident(self) -> bool:

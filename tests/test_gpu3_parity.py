@@ -414,3 +414,76 @@ def test_lattice3_launch_sweep_beside_another_cube(L, steps, eta):
     finally:
         for lat in lats:
             lat.close()
+
+
+# The launch form (mode 0), which the automatic choice keeps for large cubes, at
+# small sides: rows of whole groups and rows that groups cross, with and without
+# eta moves, a last group that is partly empty, every q kind, recorded steps, the
+# 64-bit compare, gate flips, steps of a graph and single ones.
+LAUNCHES = [
+    (2, 1, 45, 1, {}),
+    (3, 0, 70, 1, {}),
+    (4, 0, 45, 2, dict(q=2)),
+    (5, 0, 70, 3, dict(q=8)),
+    (6, 1, 45, 1, dict(init=oracle.INIT_ORDERED)),
+    (8, 1, 70, 1, dict(q=3)),
+    (9, 0, 40, 1, dict(kT=1e-3)),
+    (12, 1, 70, 7, dict(q=8)),
+    (16, 1, 40, 1, dict(kT=1e-3)),
+    (34, 1, 12, 1, {}),
+    (64, 1, 5, 1, {}),
+    (4, 1, 300, 1, dict(gates=True)),
+    (12, 1, 300, 1, dict(gates=True)),
+    (33, 0, 120, 1, dict(gates=True)),
+]
+
+
+@pytest.mark.parametrize("L,eta,steps,every,extra", LAUNCHES,
+                         ids=["L%d-%d" % (c[0], i) for i, c in enumerate(LAUNCHES)])
+def test_lattice3_launch_sweep(L, eta, steps, every, extra):
+    extra = dict(extra)
+    gates = extra.pop("gates", False)
+    if gates:
+        op = oracle.params3(L=L, seed=800 + L, kT=1.0, P=0.5, J=0.0, v_HB=0.0, epsilon=0.0,
+                            v_iso_init=1.98, dv_max_frac=0.02, eta_moves=eta)
+    elif "kT" in extra:
+        op = oracle.params3(L=L, seed=800 + L, eta_moves=eta, **extra)
+    else:
+        op = oracle.physical_params3(300.0, 0.1, L=L, seed=800 + L, dv_max_frac=0.05, eta_moves=eta, **extra)
+    ref = oracle.Oracle3(op)
+    want = ref.run(steps, every)
+    if gates:
+        gs = [r["g"] for r in want]
+        assert sum(a != b for a, b in zip(gs, gs[1:])) >= 3
+    with Lattice3(params_from_dict(asdict(op))) as lat:
+        lat.set_resident(0)
+        lat.sweep(steps // 3, every)
+        lat.sweep(steps - steps // 3, every)
+        got, overflow = lat.drain()
+        s, o, eta_got, recount = lat.state(), lat.observables(), lat.eta(), lat.recount()
+    assert not overflow and len(got) == len(want)
+    assert np.array_equal(s, ref.state())
+    assert np.array_equal(eta_got, ref.eta())
+    _same(o, ref.observables(), L)
+    assert recount == (o["n_hb_raw"], o["n_coop"])
+    for i, (g, w) in enumerate(zip(got, want)):
+        _same(g, w, ("record", i))
+
+
+@pytest.mark.parametrize("L,eta", [(16, 1), (32, 0)])
+def test_lattice3_forms_in_turn(L, eta):
+    """A run that goes through every form, one after the other, is the run of
+    any of them."""
+    op = oracle.physical_params3(300.0, 0.1, L=L, seed=9, dv_max_frac=0.05, eta_moves=eta)
+    ref = oracle.Oracle3(op)
+    with Lattice3(params_from_dict(asdict(op))) as lat:
+        for mode, steps in ((-1, 7), (0, 5), (1, 6), (0, 33), (-1, 4), (1, 3), (-1, 2)):
+            lat.set_resident(mode)
+            lat.sweep(steps, 1)
+            want = ref.run(steps, 1)
+            got, _ = lat.drain()
+            assert len(got) == len(want) == steps
+            for g, w in zip(got, want):
+                _same(g, w, (L, mode))
+        assert np.array_equal(lat.state(), ref.state())
+        assert np.array_equal(lat.eta(), ref.eta())

@@ -17,3 +17,10 @@ def test_debug_build_index_checks_hold_on_parity_cases():
                        capture_output=True, text=True, timeout=1200)
     assert r.returncode == 0, (r.stdout[-2000:], r.stderr[-4000:])
     assert "all cases match" in r.stdout
+
+
+def test_debug_build_index_checks_hold_on_further_forms():
+    r = subprocess.run([sys.executable, os.path.join(HERE, "debug_build_flow_cases.py")],
+                       capture_output=True, text=True, timeout=1200)
+    assert r.returncode == 0, (r.stdout[-2000:], r.stderr[-4000:])
+    assert "all cases match" in r.stdout
