@@ -210,9 +210,11 @@ int cvf_state_device_ptr(cvf_handle *h, void **dev_ptr);
  * get_tiles then still names the configuration of the rule for larger ones --
  * the resident form for small lattices, else the largest tile shape whose tiles
  * fill every resident block, swept as a wavefront from L = 256 up -- and the
- * larger ones run it.  The layered schedule has no tiles.  The result does not
- * depend on the config; set_tiles waits for the stream.  CVF_EINVAL for other
- * values, or a config that does not apply to the lattice. */
+ * larger ones run it.  The layered schedule has no tiles: 0, 1 and 2 all run its
+ * steps as launches, one per segment of the arm order, and -1 as one persistent
+ * launch per call (up to L = 16384).  The result does not depend on the config;
+ * set_tiles waits for the stream.  CVF_EINVAL for other values, or a config that
+ * does not apply to the lattice. */
 int cvf_set_tiles(cvf_handle *h, int32_t config);
 int cvf_get_tiles(cvf_handle *h, int32_t *config, int32_t *rows,
                   int32_t *words);

@@ -1245,8 +1245,7 @@ int cvf_set_tiles(cvf_handle* h, int32_t config) {
     const int rc = wave_scratch(h, config - kWave);
     if (rc) return rc;
   }
-  // the layered schedule has no tiles to choose
-  h->use_flow = h->flow.blocks > 0 && (config < 0 || h->p.schedule == CVF_SCHED_LAYERED);
+  h->use_flow = h->flow.blocks > 0 && config < 0;
   if (config < 0) config = auto_config(h);
   set_tile(h, config);
   return CVF_OK;

@@ -81,7 +81,8 @@ class Lattice:
         """Tile shape of the sweep (0: 64x64, 1: 32x32, 2: 16x32 words; 3: the
         whole lattice resident in one thread-block cluster; 4, 5, 6: the
         shapes of 0, 1, 2 in the wavefront sweep, one persistent launch per
-        call; -1: automatic -- up to about L = 1094 a sweep without tiles)."""
+        call; -1: automatic -- up to about L = 1094 a sweep without tiles).
+        With the layered schedule 0, 1 and 2 run launches for every step."""
         _capi.cvf_set_tiles(self.h, config)
 
     def tiles(self):

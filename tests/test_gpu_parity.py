@@ -690,3 +690,51 @@ def test_layered_series_counts_of_large_lattices(L, q, init, kT):
     assert list(records[0]["n_state"]) == list(o["n_state"])
     assert max(o["n_state"]) > 4 * L * L // 4
     assert_obs_equal(records[0], o)
+
+
+# The layered schedule's launches (a tile configuration set), which the automatic
+# choice keeps for lattices above 16384^2, at small sides.
+LAYER_LAUNCHES = [
+    (2, 80, 1, {}),
+    (8, 80, 3, dict(rng_words=2)),
+    (6, 90, 3, dict(T=270.0, init=oracle.INIT_ORDERED, q=3)),
+    (16, 90, 1, dict(T=330.0, P=50.0, q=8)),
+    (34, 30, 1, dict(rng_words=2, q=2)),
+    (66, 20, 3, dict(kT=1e-3, init=oracle.INIT_ORDERED)),
+    (64, 40, 2, dict(kT=1e-3, rng_words=2)),
+    (258, 12, 1, {}),
+    (542, 4, 1, dict(rng_words=2)),
+    (4, 300, 1, dict(gates=True)),
+    (70, 100, 1, dict(gates=True)),
+]
+
+
+@pytest.mark.parametrize("L,K,every,extra", LAYER_LAUNCHES,
+                         ids=["L%d-%d" % (c[0], i) for i, c in enumerate(LAYER_LAUNCHES)])
+def test_layered_launch_sweep(L, K, every, extra):
+    extra = dict(extra, schedule=oracle.SCHED_LAYERED)
+    if extra.pop("gates", False):
+        op = oracle.OracleParams(L=L, seed=50 + L, kT=1.0, P=0.5, J=0.0, v_HB=0.0, epsilon=0.0,
+                                 v_iso_init=1.98, dv_max_frac=0.02, **extra)
+    elif "kT" in extra:
+        op = oracle.OracleParams(L=L, seed=50 + L, **extra)
+    else:
+        T, P = extra.pop("T", 300.0), extra.pop("P", 0.1)
+        op = oracle.physical_params(T, P, L=L, seed=50 + L, dv_max_frac=0.02, **extra)
+    ref = oracle.Oracle(op)
+    want = ref.run(K, every)
+    with Lattice(params_from_dict(asdict(op))) as lat:
+        lat.set_tiles(2)
+        lat.sweep(K // 3, every)
+        lat.set_tiles(-1)              # and the persistent launch between them
+        lat.sweep(K // 3, every)
+        lat.set_tiles(0)
+        lat.sweep(K - 2 * (K // 3), every)
+        got, overflow = lat.drain()
+        s, o, counts = lat.state(), lat.observables(), lat.recount()
+    assert not overflow and len(got) == len(want)
+    assert np.array_equal(s, ref.state())
+    assert_obs_equal(o, ref.observables())
+    assert counts == (o["n_hb_raw"], o["n_coop"])
+    for i, (a, b) in enumerate(zip(got, want)):
+        assert_obs_equal(a, b, ("record", i))
