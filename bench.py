@@ -351,7 +351,7 @@ def run_kernel_mode(args):
     lat = Lattice(lib_params(cfg), stream=stream)
     if args.tiles >= 0:
         lat.set_tiles(args.tiles)
-    tiles = lat.tiles()[0]
+    tiles, form = lat.tiles()[0], lat.form()
     lat.sweep(args.warmup)
     torch.cuda.synchronize()
     ev0 = torch.cuda.Event(enable_timing=True)
@@ -363,7 +363,7 @@ def run_kernel_mode(args):
     ms = ev0.elapsed_time(ev1)
     o = lat.observables()
     lat.close()
-    print(json.dumps({"mode": "kernel", "L": args.L, "tiles": tiles, "sweeps": args.steps, "ms": ms,
+    print(json.dumps({"mode": "kernel", "L": args.L, "tiles": tiles, "form": form, "sweeps": args.steps, "ms": ms,
                       "updates_per_ns": 4.0 * args.L * args.L * args.steps / (ms * 1e6),
                       "n_hb_raw": o["n_hb_raw"], "n_coop": o["n_coop"]}))
     return 0
@@ -664,14 +664,15 @@ def measure_batched(args, rank):
 
     def solo(resident_ok):
         """The replicas one at a time through the single-lattice API: with
-        resident_ok, each in its fastest form (small lattices stay in one
-        cluster for all the steps); without, one launch per MC step."""
+        resident_ok, each in its automatic form (one launch for all the
+        steps); without, the tiled sweep (one launch per MC step)."""
         total_ms = 0.0
         with torch.cuda.stream(stream):
             for p in ps:
                 with Lattice(p, stream=stream) as lat:
-                    if not resident_ok and lat.tiles()[0] == 3:
+                    if not resident_ok:
                         lat.set_tiles(2)
+                        assert lat.form() == "launches"
                     lat.sweep(3)
                     torch.cuda.synchronize()
                     e0 = torch.cuda.Event(enable_timing=True)
@@ -694,8 +695,8 @@ def measure_batched(args, rank):
             "speedup_vs_one_replica_per_launch": batched_rate / per_launch_rate,
             "one_lattice_at_a_time": {"value": alone_rate, "unit": "replica-sweeps/s",
                                       "sweeps_each": solo_steps,
-                                      "form": "each replica alone in its fastest single-lattice "
-                                              "form (small lattices resident in one cluster)"},
+                                      "form": "each replica alone in its automatic single-lattice "
+                                              "form (one launch for all the steps)"},
             "speedup_vs_one_lattice_at_a_time": batched_rate / alone_rate,
             "tile_config": best, "tile": list(tile_configs()[best][:2]),
             "block_threads": tile_configs()[best][2],
@@ -810,15 +811,17 @@ def main():
     value = updates / (dev_s * 1e9)
     obs = [l.observables() for l in lats]
 
-    # dominant kernel: the sweep of the automatic configuration (at 4096^2
-    # the wavefront, k_sweep_wave: one launch per call; the tiled sweep:
-    # one launch per MC step); its time per MC step from CUDA events around
+    # dominant kernel: the sweep of the form that runs (at 4096^2 the
+    # wavefront, k_sweep_wave: one launch per call); its time per MC step from
+    # CUDA events around
     # a 200-step call on the lattice's stream
     sw_ms = []
     lat = lats[1]
-    wave = lat.tiles()[0] >= 4
-    sweep_kernel = ("k_sweep_wave (one launch per call, the MC steps of the call in a wavefront)"
-                    if wave else "k_sweep_tiled (one launch per MC step)")
+    form = lat.form()
+    sweep_kernel = {"wavefront": "k_sweep_wave (one launch per call, the MC steps of the call in a wavefront)",
+                    "dataflow": "k_flow2 (one launch per call, every word with its own progress)",
+                    "cluster": "k_resident2 (one launch per call, the lattice in one cluster)",
+                    "launches": "k_sweep_tiled (one launch per MC step)"}[form]
     for _ in range(5):
         ev0 = torch.cuda.Event(enable_timing=True)
         ev1 = torch.cuda.Event(enable_timing=True)
@@ -915,9 +918,10 @@ def main():
                     small[k]["oracle"] = v
             except Exception as e:
                 small["oracle_error"] = str(e)
-        # k_set_record per call, then one k_sweep_wave launch per call or one
-        # k_sweep_tiled launch per MC step (the volume move runs inside it)
-        launches_per_call = 2 if wave else S + 1
+        # one k_flow2 launch per call, or k_set_record and then one k_sweep_wave
+        # (k_resident2) launch per call or one k_sweep_tiled launch per MC step
+        # (the volume move runs inside each)
+        launches_per_call = {"dataflow": 1, "launches": S + 1}.get(form, 2)
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": dev_s * 1e3 / args.steps, "higher_is_better": True,

@@ -219,6 +219,17 @@ int cvf_set_tiles(cvf_handle *h, int32_t config);
 int cvf_get_tiles(cvf_handle *h, int32_t *config, int32_t *rows,
                   int32_t *words);
 
+/* The form that the handle's next sweep runs as (cvf_get_form, cvf3_get_form),
+ * or that a batch's last one ran as (cvf_batch_get_form; -1 before any).  The
+ * settings above and below name a rule's choice, which the dataflow sweep takes
+ * the place of where it applies. */
+#define CVF_FORM_LAUNCHES 0  /* one or more launches for every step */
+#define CVF_FORM_CLUSTER 1   /* one launch per call, the lattice in one cluster's shared memory */
+#define CVF_FORM_WAVEFRONT 2 /* one launch per call, tiles that wait for those around them */
+#define CVF_FORM_DATAFLOW 3  /* one launch per call, every word with its own progress */
+#define CVF_FORM_TILE_QUEUE 4 /* batch: one launch per call, tiles of all replicas in turn */
+int cvf_get_form(cvf_handle *h, int32_t *form);
+
 /* Waits for the handle's stream, frees what the library allocated. */
 int cvf_destroy(cvf_handle *h);
 
@@ -348,6 +359,7 @@ int cvf_batch_get_state(cvf_batch *b, int32_t replica, uint16_t *host,
  * configuration that the last call's rule chose (-1 before any call). */
 int cvf_batch_set_tiles(cvf_batch *b, int32_t config);
 int cvf_batch_get_tiles(cvf_batch *b, int32_t *config, int32_t *last_used);
+int cvf_batch_get_form(cvf_batch *b, int32_t *form);
 int cvf_batch_tile_config(int32_t config, int32_t *rows, int32_t *words);
 int cvf_batch_config_threads(int32_t config, int32_t *threads);
 
@@ -489,6 +501,7 @@ int cvf3_state_device_ptr(cvf3_handle *h, void **dev_ptr);
  * small cubes that mode 1 takes (up to 24, and 32 with a 16-CTA cluster). */
 int cvf3_set_resident(cvf3_handle *h, int32_t mode);
 int cvf3_get_resident(cvf3_handle *h, int32_t *resident);
+int cvf3_get_form(cvf3_handle *h, int32_t *form); /* CVF_FORM_* */
 
 /* Waits for the handle's stream, frees what the library allocated. */
 int cvf3_destroy(cvf3_handle *h);

@@ -75,6 +75,7 @@ _SIGS = {
     "cvf_destroy": (ctypes.c_int, [_vp]),
     "cvf_set_tiles": (ctypes.c_int, [_vp, ctypes.c_int32]),
     "cvf_get_tiles": (ctypes.c_int, [_vp, _P(ctypes.c_int32), _P(ctypes.c_int32), _P(ctypes.c_int32)]),
+    "cvf_get_form": (ctypes.c_int, [_vp, _P(ctypes.c_int32)]),
     "cvf_philox_probe": (ctypes.c_int, [ctypes.c_uint64, ctypes.c_uint32, ctypes.c_int64, _vp, _vp]),
     "cvf_sweep_noalloc": (ctypes.c_int, [_P(cvf_params), _vp, ctypes.c_double, ctypes.c_int64,
                                          ctypes.c_int64, ctypes.c_int32, _P(cvf_obs), ctypes.c_int64,
@@ -96,6 +97,7 @@ _SIGS = {
     "cvf_batch_get_state": (ctypes.c_int, [_vp, ctypes.c_int32, _P(ctypes.c_uint16), ctypes.c_size_t]),
     "cvf_batch_set_tiles": (ctypes.c_int, [_vp, ctypes.c_int32]),
     "cvf_batch_get_tiles": (ctypes.c_int, [_vp, _P(ctypes.c_int32), _P(ctypes.c_int32)]),
+    "cvf_batch_get_form": (ctypes.c_int, [_vp, _P(ctypes.c_int32)]),
     "cvf_batch_tile_config": (ctypes.c_int, [ctypes.c_int32, _P(ctypes.c_int32), _P(ctypes.c_int32)]),
     "cvf_batch_config_threads": (ctypes.c_int, [ctypes.c_int32, _P(ctypes.c_int32)]),
     "cvf_batch_destroy": (ctypes.c_int, [_vp]),
@@ -116,6 +118,7 @@ _SIGS = {
     "cvf3_destroy": (ctypes.c_int, [_vp]),
     "cvf3_set_resident": (ctypes.c_int, [_vp, ctypes.c_int32]),
     "cvf3_get_resident": (ctypes.c_int, [_vp, _P(ctypes.c_int32)]),
+    "cvf3_get_form": (ctypes.c_int, [_vp, _P(ctypes.c_int32)]),
     "cvf_get_window": (ctypes.c_int, [_vp, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32,
                                       ctypes.c_int32, _P(ctypes.c_uint16)]),
     "cvf3_get_window": (ctypes.c_int, [_vp] + [ctypes.c_int32] * 6 + [_P(ctypes.c_uint32)]),
@@ -244,6 +247,28 @@ def cvf_get_tiles(h: int):
     _check(load().cvf_get_tiles(h, ctypes.byref(c), ctypes.byref(r), ctypes.byref(w)),
            "cvf_get_tiles")
     return c.value, r.value, w.value
+
+
+# names of CVF_FORM_*
+FORMS = ("launches", "cluster", "wavefront", "dataflow", "tile queue")
+
+
+def _form(name: str, handle: int):
+    f = ctypes.c_int32()
+    _check(getattr(load(), name)(handle, ctypes.byref(f)), name)
+    return FORMS[f.value] if f.value >= 0 else None
+
+
+def cvf_get_form(h: int) -> str:
+    return _form("cvf_get_form", h)
+
+
+def cvf_batch_get_form(b: int):
+    return _form("cvf_batch_get_form", b)
+
+
+def cvf3_get_form(h: int) -> str:
+    return _form("cvf3_get_form", h)
 
 
 def cvf_sweep_noalloc(p: cvf_params, dev_state: int, V_iso: float, sweep: int, n_sweeps: int,

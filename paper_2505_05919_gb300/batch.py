@@ -75,8 +75,13 @@ class Batch:
         _capi.cvf_batch_set_tiles(self.b, config)
 
     def tiles(self) -> tuple:
-        """(setting, configuration the last call used)."""
+        """(setting, configuration the last call's rule chose)."""
         return _capi.cvf_batch_get_tiles(self.b)
+
+    def form(self):
+        """What the last call ran as: "tile queue", "dataflow", or None before
+        any."""
+        return _capi.cvf_batch_get_form(self.b)
 
     # results ---------------------------------------------------------------
     def observables(self, rid: int) -> dict:

@@ -1446,6 +1446,12 @@ int cvf3_get_resident(cvf3_handle* h, int32_t* resident) {
   return CVF_OK;
 }
 
+int cvf3_get_form(cvf3_handle* h, int32_t* form) {
+  if (!h || !form) return set_error(CVF_EINVAL, "NULL argument");
+  *form = h->cluster ? CVF_FORM_CLUSTER : h->use_flow ? CVF_FORM_DATAFLOW : CVF_FORM_LAUNCHES;
+  return CVF_OK;
+}
+
 int cvf3_state_device_ptr(cvf3_handle* h, void** dev_ptr) {
   if (!h || !dev_ptr) return set_error(CVF_EINVAL, "NULL argument");
   *dev_ptr = h->state;

@@ -106,7 +106,8 @@ struct cvf_batch {
   int rng_words;       // shared by all replicas (-1 while empty)
   int kernel_words;    // the one whose kernels graph, grid and flow_slots are of
   int tile_cfg;        // -1: chosen per call
-  int last_cfg;        // the shape the last call used
+  int last_cfg;        // the shape the last call's rule chose
+  int last_form;       // CVF_FORM_* of the last call
   ReplicaDesc* d_reps;
   int d_reps_cap;
   bool reps_dirty;
@@ -456,6 +457,7 @@ int cvf_batch_create(const cvf_params* params, int32_t n, void* stream, cvf_batc
   b->kernel_words = -1;
   b->tile_cfg = -1;
   b->last_cfg = -1;
+  b->last_form = -1;
   cudaError_t e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) {
     int dev = 0;
@@ -623,6 +625,12 @@ int cvf_batch_get_tiles(cvf_batch* b, int32_t* config, int32_t* last_used) {
   return CVF_OK;
 }
 
+int cvf_batch_get_form(cvf_batch* b, int32_t* form) {
+  if (!b || !form) return set_error(CVF_EINVAL, "NULL argument");
+  *form = b->last_form;
+  return CVF_OK;
+}
+
 int cvf_batch_tile_config(int32_t config, int32_t* rows, int32_t* words) {
   if (config < 0 || config >= kNumTileConfigs || !rows || !words)
     return set_error(CVF_EINVAL, "tile config %d (0..%d)", config, kNumTileConfigs - 1);
@@ -683,6 +691,7 @@ int cvf_batch_sweep(cvf_batch* b, const int64_t* sweeps, int32_t n) {
     rc = flow_sweep(b, act, sweeps, any_cmp64(b), &done);
     if (rc) return rc;
     if (done) {
+      b->last_form = CVF_FORM_DATAFLOW;
       for (int i : act) b->reps[i].sweep_host += sweeps[i];
       return CVF_OK;
     }
@@ -720,6 +729,7 @@ int cvf_batch_sweep(cvf_batch* b, const int64_t* sweeps, int32_t n) {
   CVF_CUDA_CHECK(cudaEventRecord(b->ev_work[slot], b->stream));
   rc = launch(b, cfg, any_cmp64(b), n, na);
   if (rc) return rc;
+  b->last_form = CVF_FORM_TILE_QUEUE;
   for (int i : act) b->reps[i].sweep_host += sweeps[i];
   return CVF_OK;
 }

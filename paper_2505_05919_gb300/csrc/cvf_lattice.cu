@@ -1261,6 +1261,15 @@ int cvf_get_tiles(cvf_handle* h, int32_t* config, int32_t* rows, int32_t* words)
   return CVF_OK;
 }
 
+int cvf_get_form(cvf_handle* h, int32_t* form) {
+  if (!h || !form) return set_error(CVF_EINVAL, "NULL argument");
+  *form = h->use_flow                                                        ? CVF_FORM_DATAFLOW
+          : is_wave(h->tile)                                                 ? CVF_FORM_WAVEFRONT
+          : h->tile == kResident && h->p.schedule == CVF_SCHED_CHECKERBOARD ? CVF_FORM_CLUSTER
+                                                                             : CVF_FORM_LAUNCHES;
+  return CVF_OK;
+}
+
 int cvf_destroy(cvf_handle* h) {
   if (!h) return CVF_OK;
   cudaError_t e = cudaStreamSynchronize(h->stream);

@@ -90,6 +90,11 @@ class Lattice:
         choice the rule's, also where the lattice runs without tiles)."""
         return _capi.cvf_get_tiles(self.h)
 
+    def form(self) -> str:
+        """What a sweep runs as: "launches" (of every step), "cluster",
+        "wavefront" or "dataflow" (one launch per call each)."""
+        return _capi.cvf_get_form(self.h)
+
     def close(self) -> None:
         if getattr(self, "h", None):
             _capi.cvf_destroy(self.h)

@@ -91,7 +91,14 @@ class Lattice3:
         _capi.cvf3_set_resident(self.h, mode)
 
     def resident(self) -> bool:
+        """Whether the setting or its rule names the cluster (form() says what
+        runs)."""
         return bool(_capi.cvf3_get_resident(self.h))
+
+    def form(self) -> str:
+        """What a sweep runs as: "launches" (of every step), "cluster" or
+        "dataflow" (one launch per call each)."""
+        return _capi.cvf3_get_form(self.h)
 
     def close(self) -> None:
         if getattr(self, "h", None):

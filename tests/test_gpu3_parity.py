@@ -487,3 +487,12 @@ def test_lattice3_forms_in_turn(L, eta):
                 _same(g, w, (L, mode))
         assert np.array_equal(lat.state(), ref.state())
         assert np.array_equal(lat.eta(), ref.eta())
+
+
+def test_lattice3_the_form_that_runs_is_reported():
+    for L, eta, mode, form in ((16, 1, -1, "dataflow"), (16, 1, 0, "launches"), (16, 1, 1, "cluster"),
+                               (40, 1, -1, "dataflow"), (128, 1, -1, "dataflow"), (130, 1, -1, "launches"),
+                               (111, 0, -1, "dataflow"), (113, 0, -1, "launches"), (9, 0, 0, "launches")):
+        with Lattice3(params_from_dict(asdict(oracle.physical_params3(300.0, 0.1, L=L, eta_moves=eta)))) as lat:
+            lat.set_resident(mode)
+            assert lat.form() == form, (L, eta, mode)

@@ -334,3 +334,16 @@ def test_batch_emptied_and_refilled_with_other_draws(first, then, cfg):
         want, ow = _solo(p, [6])
         assert np.array_equal(s, want), (p.L, cfg)
         _same(o, ow)
+
+
+def test_batch_the_form_that_ran_is_reported():
+    with Batch([_params(L, seed=L) for L in (64, 32)]) as b:
+        assert b.form() is None
+        b.sweep([3, 2])
+        assert b.form() == "dataflow" and b.tiles() == (-1, 11)
+        b.set_tiles(3)
+        b.sweep([3, 2])
+        assert b.form() == "tile queue" and b.tiles() == (3, 3)
+    with Batch([_params(1024, seed=5), _params(512, seed=6)]) as b:   # more than the dataflow launch holds
+        b.sweep([2, 2])
+        assert b.form() == "tile queue"

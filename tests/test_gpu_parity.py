@@ -738,3 +738,21 @@ def test_layered_launch_sweep(L, K, every, extra):
     assert counts == (o["n_hb_raw"], o["n_coop"])
     for i, (a, b) in enumerate(zip(got, want)):
         assert_obs_equal(a, b, ("record", i))
+
+
+def test_the_form_that_runs_is_reported():
+    """form() names the kernels of the next sweep, also where tiles() names the
+    configuration of a rule that the dataflow sweep takes the place of."""
+    layered = oracle.SCHED_LAYERED
+    for L, schedule, config, form in ((64, 0, -1, "dataflow"), (64, 0, 3, "cluster"), (64, 0, 2, "launches"),
+                                      (1024, 0, -1, "dataflow"), (1024, 0, 6, "wavefront"),
+                                      (1024, 0, 0, "launches"), (2048, 0, -1, "wavefront"),
+                                      (64, layered, -1, "dataflow"), (64, layered, 0, "launches")):
+        with Lattice(params(300.0, 0.1, L=L, schedule=schedule)) as lat:
+            assert lat.form() == ("wavefront" if L == 2048 else "dataflow")
+            lat.set_tiles(config)
+            assert lat.form() == form, (L, schedule, config)
+            if config >= 0:
+                assert lat.tiles()[0] == config
+            lat.set_tiles(-1)
+            assert lat.form() == ("wavefront" if L == 2048 else "dataflow")
