@@ -14,7 +14,12 @@ tile's work (a small lattice's step is a chain of such tiles).
 For a list of replica parameters the tuner builds a scratch batch with the
 same lattice sizes (other seeds, so the caller's replicas are untouched),
 times a short probe on every configuration with CUDA events, and returns
-the fastest.  Results are cached for the process by the mix of (L, q,
+the fastest.  The automatic setting (-1) is not a configuration: where all
+replicas are resident at once (up to about 1.2 million cells in at most 128
+replicas) it runs without tiles and is faster than each of them (24 lattices of
+64^2: 2.2 us per step against 8.9), and a configuration that is set switches
+that off.  With ``automatic=True`` it is probed as well, and -1 is returned
+where it wins.  Results are cached for the process by the mix of (L, q,
 rng_words) and the probe length.  The state points (T, P) are not part of
 the key: an arm update's accept or reject is a predicated select, so a
 cell costs the same at any acceptance rate (the batched workload's sizes
@@ -37,15 +42,18 @@ def signature(params_list) -> tuple:
 
 
 def cells_per_thread(config: int) -> int:
-    """Cells one of the block's 256 threads updates per MC step."""
+    """Cells one of the block's threads updates per MC step."""
+    if config < 0:
+        raise ValueError("the automatic setting has no tile of its own")
     rows, words, threads = tile_configs()[config]
     return 2 * rows * words // threads
 
 
-def autotune(params_list, probe_sweeps: int = 20, warmup: int = 3, stream=None):
-    """Returns (best_config, {config: ms_per_step})."""
+def autotune(params_list, probe_sweeps: int = 20, warmup: int = 3, stream=None, automatic: bool = False):
+    """Returns (best_config, {config: ms_per_step}) over the tile
+    configurations and, with automatic, the automatic setting -1."""
     import torch
-    key = (signature(params_list), probe_sweeps)
+    key = (signature(params_list), probe_sweeps, automatic)
     if key in _cache:
         return _cache[key]
     scratch = []
@@ -57,7 +65,7 @@ def autotune(params_list, probe_sweeps: int = 20, warmup: int = 3, stream=None):
     timings = {}
     with Batch(scratch, stream=stream) as b:
         n = b.slots()
-        for cfg in range(len(tile_configs())):
+        for cfg in ([-1] if automatic else []) + list(range(len(tile_configs()))):
             b.set_tiles(cfg)
             b.sweep([warmup] * n)
             b.sync()

@@ -113,3 +113,15 @@ def test_cells_per_thread_follows_the_configuration():
     for c, (rows, words, threads) in enumerate(tile_configs()):
         assert AT.cells_per_thread(c) == 2 * rows * words // threads
     assert AT.cells_per_thread(0) == 32        # 64 x 64 words, 256 threads
+
+
+def test_the_automatic_setting_is_probed_when_asked_for(fakes):
+    COST[-1] = 0.2
+    COST[7] = 0.5
+    assert AT.autotune(reps(), probe_sweeps=20)[0] == 7         # tile configurations only
+    best, t = AT.autotune(reps(), probe_sweeps=20, automatic=True)
+    assert best == -1 and set(t) == {-1} | set(range(len(tile_configs())))
+    COST[-1] = 0.9
+    assert AT.autotune(reps(sizes=(32, 64)), probe_sweeps=20, automatic=True)[0] == 7
+    with pytest.raises(ValueError):
+        AT.cells_per_thread(-1)

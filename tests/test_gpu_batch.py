@@ -347,3 +347,14 @@ def test_batch_the_form_that_ran_is_reported():
     with Batch([_params(1024, seed=5), _params(512, seed=6)]) as b:   # more than the dataflow launch holds
         b.sweep([2, 2])
         assert b.form() == "tile queue"
+
+
+def test_autotuner_with_the_automatic_setting():
+    # 24 of 64^2: without tiles a step takes a quarter of the fastest tile's
+    ps = [_params(64, seed=i) for i in range(24)]
+    best, timings = autotune.autotune(ps, probe_sweeps=200, automatic=True)
+    assert best == -1 and set(timings) == {-1} | set(range(len(tile_configs())))
+    with Batch(ps) as b:
+        b.set_tiles(best)
+        b.sweep([2] * len(ps))
+        assert b.form() == "dataflow"
