@@ -214,7 +214,12 @@ int cvf_state_device_ptr(cvf_handle *h, void **dev_ptr);
  * steps as launches, one per segment of the arm order, and -1 as one persistent
  * launch per call (up to L = 16384).  The result does not depend on the config;
  * set_tiles waits for the stream.  CVF_EINVAL for other values, or a config that
- * does not apply to the lattice. */
+ * does not apply to the lattice.
+ * Lattices on streams of their own: one up to 128^2 takes at most 16 SMs; several
+ * up to about 260^2 (cubes up to 36^3) run beside each other on all of them; a
+ * larger one that runs without tiles holds every SM until its call is done, so
+ * that calls on several streams take turns (a batch runs such replicas in one
+ * launch). */
 int cvf_set_tiles(cvf_handle *h, int32_t config);
 int cvf_get_tiles(cvf_handle *h, int32_t *config, int32_t *rows,
                   int32_t *words);

@@ -97,8 +97,9 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
     flow_books(A, U.vol, H, (int)gridDim.x - 1, copy, end_tag, step0, n_steps, every, err);
     return;
   }
-  constexpr int kFlowThreads = ONE ? kFlowThreadsOne : kFlowThreadsMany;
-  constexpr int kFlowBlock = kFlowThreads + 32;
+  // sweeping threads; the warp after them is the clerk
+  const uint32_t sweepers = ONE ? blockDim.x - 32u : (uint32_t)kFlowThreadsMany;
+  const int threads = (int)sweepers + 32;
   FlowSmem& S = U.sweep;
   const uint32_t b = blockIdx.x - 1u;
   uint32_t* const F = copy + kFlowHead;             // the cells' words
@@ -111,15 +112,16 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
   // them (70^3 without eta moves 22.3 us per step, so 14.0; 97^3 38.1 / 26.2).
   // From four rounds of aligned groups on the idle warps cost more (100^3 19.5
   // us with all of them, 21.9 so).
-  const uint32_t rounds = (groups_per_block + kFlowThreads - 1u) / kFlowThreads;
-  const uint32_t stride = (ALIGNED && rounds > 3u)
-                              ? (uint32_t)kFlowThreads
+  const uint32_t rounds = (groups_per_block + sweepers - 1u) / sweepers;
+  const uint32_t stride = ONE ? (uint32_t)kFlowThreadsOne  // (no second round)
+                          : (ALIGNED && rounds > 3u)
+                              ? sweepers
                               : (groups_per_block / 32u + rounds - 1u) / rounds * 32u;
   const int warps = (int)min((g_hi - g_lo + 31u) / 32u, stride / 32u);  // that have a group
   const uint32_t q = A.q;
-  for (int g = 0; g < 2; ++g) fill_rows3(S.Tb[g], A.table + g * kRows3, kFlowBlock);
-  fill_prop3(S.Tb[0], q, kFlowBlock);
-  fill_prop3(S.Tb[1], q, kFlowBlock);
+  for (int g = 0; g < 2; ++g) fill_rows3(S.Tb[g], A.table + g * kRows3, threads);
+  fill_prop3(S.Tb[0], q, threads);
+  fill_prop3(S.Tb[1], q, threads);
   if (eta_on && threadIdx.x < 18) S.eta_thr[threadIdx.x / 9][threadIdx.x % 9] = A.eta_table[threadIdx.x];
   if (eta_on && threadIdx.x < 9) {
     const uint32_t m = A.masks[threadIdx.x];
@@ -136,10 +138,10 @@ __global__ void __launch_bounds__((ONE ? kFlowThreadsOne : kFlowThreadsMany) + 3
   }
   {
     uint32_t* ring = reinterpret_cast<uint32_t*>(S.ring);
-    for (int i = threadIdx.x; i < (int)(sizeof(S.ring) / 4); i += kFlowBlock) ring[i] = 0u;
+    for (int i = threadIdx.x; i < (int)(sizeof(S.ring) / 4); i += threads) ring[i] = 0u;
   }
   __syncthreads();
-  if (threadIdx.x >= kFlowThreads) {
+  if (threadIdx.x >= sweepers) {
     flow_clerk([&](long long s) { return make_plan(s, A.keys); }, S.ring, warps, H, err, step0,
                n_steps, every);
     return;
@@ -456,6 +458,7 @@ Flow3Plan flow3_plan(const Args3& A, bool cmp64) {
     if (room < 1 || (one && groups > room * flow_threads(true))) continue;
     const long long share = (groups + room - 1) / room;
     P.groups_per_block = (uint32_t)((share + 31) / 32 * 32);
+    if (one) P.threads = flow_block(P.kernel, P.groups_per_block, P.threads);
     P.blocks = (int)((groups + P.groups_per_block - 1) / P.groups_per_block);
   }
   P.copy_words = (size_t)kFlowHead + 4 * (size_t)groups + A.ncube;

@@ -135,12 +135,13 @@ __device__ __forceinline__ CellWords<RNG_WORDS> cell_words(uint32_t c, const Ste
 
 // A block of a lattice's launch: the books (b < 0) or block b of `blocks` that
 // sweep.
-template <int RNG_WORDS, bool CMP64, int V, int NT>
+template <int RNG_WORDS, bool CMP64, int V>
 __device__ __forceinline__ void flow2_strips(Flow2Block& U, const LatticeArgs& A,
                                              const Flow2Geom& G, WaveHdr* H, uint32_t* copy,
                                              long long n_steps, int every, int b, int blocks,
                                              unsigned int* err) {
   constexpr bool kAhead = V <= kAheadRows;  // the draws of a part are made before its loads
+  const int sweepers = (int)blockDim.x - 32;  // threads; the last warp is the clerk
   Ctrl* const ctl = A.ctrl;
   // the committed step count and the copy's tag: neither changes before every
   // block has taken part in the first (last) step
@@ -156,9 +157,9 @@ __device__ __forceinline__ void flow2_strips(Flow2Block& U, const LatticeArgs& A
   uint32_t* const F = copy + kFlow2Head;
   const uint32_t t_lo = (uint32_t)b * G.per_block, t_hi = min(t_lo + G.per_block, G.items);
   const int warps = (int)((t_hi - t_lo + 31u) / 32u);
-  flow2_setup(S, A, NT + 32);
+  flow2_setup(S, A, (int)blockDim.x);
   __syncthreads();
-  if (threadIdx.x >= NT) {
+  if ((int)threadIdx.x >= sweepers) {
     flow_clerk([](long long) { return 0ull; }, S.ring, warps, H, err, step0, n_steps, every);
     return;
   }
@@ -305,8 +306,8 @@ __global__ void __launch_bounds__(NT + 32, 1)
     k_flow2(const __grid_constant__ LatticeArgs A, const __grid_constant__ Flow2Geom G, WaveHdr* H,
             uint32_t* copy, long long n_steps, int every) {
   __shared__ Flow2Block U;
-  flow2_strips<RNG_WORDS, CMP64, V, NT>(U, A, G, H, copy, n_steps, every, (int)blockIdx.x - 1,
-                                        (int)gridDim.x - 1, &A.ctrl->error);
+  flow2_strips<RNG_WORDS, CMP64, V>(U, A, G, H, copy, n_steps, every, (int)blockIdx.x - 1,
+                                    (int)gridDim.x - 1, &A.ctrl->error);
 }
 
 // Many lattices, each with blocks of its own and its own number of steps: the
@@ -317,7 +318,7 @@ __global__ void __launch_bounds__(NT + 32, 1024 / (NT + 32))
     k_flow2_batch(const __grid_constant__ Flow2Batch B) {
   __shared__ Flow2Block U;
   const Flow2Replica& R = B.item[B.of_block[blockIdx.x]];
-  flow2_strips<RNG_WORDS, CMP64, V, NT>(
+  flow2_strips<RNG_WORDS, CMP64, V>(
       U, R.args, R.geom, R.hdr, R.copy, R.n_steps, 0,
       blockIdx.x < (unsigned int)B.n ? -1 : (int)(blockIdx.x - R.first_block), (int)R.blocks,
       B.err);
@@ -504,12 +505,14 @@ __global__ void __launch_bounds__(NT + 32, 1)
   uint32_t* const F = copy + kFlow2Head;
   const uint32_t t_lo = (blockIdx.x - 1u) * G.per_block, t_hi = min(t_lo + G.per_block, G.items);
   // as many groups for every warp, as in the cubic sweep
-  const uint32_t rounds = (G.per_block + NT - 1u) / NT;
-  const uint32_t stride = (G.per_block / 32u + rounds - 1u) / rounds * 32u;
+  // sweeping threads; the warp after them is the clerk
+  const uint32_t sweepers = ONE ? blockDim.x - 32u : (uint32_t)NT;
+  const uint32_t rounds = (G.per_block + sweepers - 1u) / sweepers;
+  const uint32_t stride = ONE ? (uint32_t)NT : (G.per_block / 32u + rounds - 1u) / rounds * 32u;
   const int warps = (int)min((t_hi - t_lo + 31u) / 32u, stride / 32u);
-  flow2_setup(S, A, NT + 32);
+  flow2_setup(S, A, (int)sweepers + 32);
   __syncthreads();
-  if (threadIdx.x >= NT) {
+  if (threadIdx.x >= sweepers) {
     flow_clerk([&](long long s) { return (unsigned long long)layer_plan(s, A.keys); }, S.ring,
                warps, H, err, step0, n_steps, every);
     return;
@@ -708,7 +711,7 @@ bool adopt(Flow2Plan* P, const Flow2Form& form, int rng_words, bool cmp64, long 
   if (room < 1 || (one && items > room * form.threads)) return false;
   const long long share = ((items + room - 1) / room + 31) / 32 * 32;
   P->kernel = kernel;
-  P->threads = form.threads + 32;
+  P->threads = one ? flow_block(kernel, share, form.threads + 32) : form.threads + 32;
   P->geom.items = (uint32_t)items;
   P->geom.per_block = (uint32_t)share;
   P->blocks = (int)((items + share - 1) / share);

@@ -496,3 +496,24 @@ def test_lattice3_the_form_that_runs_is_reported():
         with Lattice3(params_from_dict(asdict(oracle.physical_params3(300.0, 0.1, L=L, eta_moves=eta)))) as lat:
             lat.set_resident(mode)
             assert lat.form() == form, (L, eta, mode)
+
+
+@pytest.mark.parametrize("L,n,eta", [(6, 6, 1), (16, 8, 1), (33, 4, 0), (32, 4, 1), (44, 3, 1)])
+def test_lattice3_cubes_beside_each_other(L, n, eta):
+    import torch
+    ops = [oracle.physical_params3(300.0, 0.1, L=L, seed=20 + i, dv_max_frac=0.05, eta_moves=eta) for i in range(n)]
+    streams = [torch.cuda.Stream() for _ in ops]
+    lats = [Lattice3(params_from_dict(asdict(op)), stream=s) for op, s in zip(ops, streams)]
+    try:
+        for steps in (1, 8, 3):
+            for lat in lats:
+                lat.sweep(steps)
+        for op, lat in zip(ops, lats):
+            ref = oracle.Oracle3(op)
+            ref.run(12)
+            assert np.array_equal(lat.state(), ref.state())
+            assert np.array_equal(lat.eta(), ref.eta())
+            _same(lat.observables(), ref.observables(), L)
+    finally:
+        for lat in lats:
+            lat.close()

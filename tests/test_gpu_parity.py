@@ -756,3 +756,29 @@ def test_the_form_that_runs_is_reported():
                 assert lat.tiles()[0] == config
             lat.set_tiles(-1)
             assert lat.form() == ("wavefront" if L == 2048 else "dataflow")
+
+
+@pytest.mark.parametrize("L,n,extra", [(130, 8, {}), (258, 4, dict(rng_words=2)), (64, 8, dict(schedule=oracle.SCHED_LAYERED)),
+                                       (66, 8, {}), (382, 3, {})])
+def test_lattices_beside_each_other(L, n, extra):
+    """Lattices on streams of their own, several of whose persistent launches are
+    on the GPU at once, each end as the oracle's."""
+    import torch
+    ops = [oracle.physical_params(300.0, 0.1, L=L, seed=70 + i, dv_max_frac=0.02, **extra) for i in range(n)]
+    streams = [torch.cuda.Stream() for _ in ops]
+    lats = [Lattice(params_from_dict(asdict(op)), stream=s) for op, s in zip(ops, streams)]
+    try:
+        for steps in (1, 12, 7):
+            for lat in lats:
+                lat.sweep(steps, 3)
+        for op, lat in zip(ops, lats):
+            s, o, records = oracle_run(op, 20, record_every=3)
+            assert np.array_equal(lat.state(), s)
+            assert_obs_equal(lat.observables(), o)
+            got, _ = lat.drain()
+            assert len(got) == len(records)
+            for a, b in zip(got, records):
+                assert_obs_equal(a, b)
+    finally:
+        for lat in lats:
+            lat.close()
