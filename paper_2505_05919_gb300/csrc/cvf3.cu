@@ -50,13 +50,13 @@ constexpr long long kRingCap3 = 65536;
 constexpr int kMaxSide3 = 1024;
 // The dataflow sweep (cvf3_flow.cu) takes cubes of up to this many groups
 // (128^3): there it still beats four launches per step, us per MC step with
-// the eta update: 16^3 4.0 against 14.6, 32^3 4.0 / 15.7, 64^3 8.0 / 17.0,
-// 100^3 22.4 / 29.9, 128^3 43.9 / 48.2, but 144^3 61.1 / 58.0 and 260^3 375 /
-// 271: it looks at every word's tag, and sixteen warps of an SM hide less
+// the eta update: 16^3 4.0 against 15.1, 32^3 4.0 / 15.6, 64^3 7.5 to 8.2 / 17.2,
+// 100^3 22.1 / 29.1, 128^3 43.8 / 45.8, but 144^3 61.1 / 57.4 and 260^3 375 /
+// 272: it looks at every word's tag, and sixteen warps of an SM hide less
 // latency than the launches' thirty-two.  Without the eta update and with rows
 // that are no whole groups, where a word is a load of its own, up to 112^3
-// (51^3 5.7 / 16.0, 73^3 16.7 / 19.9, 97^3 26.2 / 33.4, 109^3 38.2 / 41.8, but
-// 115^3 45.5 / 43.6).
+// (51^3 5.8 / 16.4, 73^3 17.7 / 20.1, 97^3 29.2 / 31.9, about even at 109^3 with
+// 40.5 / 39.2, but 115^3 45.5 / 43.9).
 constexpr uint32_t kFlowMaxGroups = 1u << 19;
 constexpr uint32_t kFlowMaxGroupsRagged = 112u * 112u * 112u / 4u;
 
@@ -489,9 +489,10 @@ __global__ void __launch_bounds__(kThreads3) k_eta_bits3(Args3 A) {
 // shared memory.  Every cell is updated with the same draws and rule as in
 // k_pass3, so the results are identical.  512 threads give every group a
 // thread up to 32^3 (256 took two rounds: 32^3 12.2 against 8.8 us per step,
-// 24^3 11.7 / 8.6).  Two more warps of CTA 0 decide the next step's volume move, overlapping the first segment; CTA 0 commits the
-// step after the last segment.  All CTAs follow the same plan (computed from
-// the step by each), so they meet the same barriers.
+// 24^3 11.7 / 8.6).  Two more warps of CTA 0 decide the next step's volume move,
+// overlapping the first segment; CTA 0 commits the step after the last segment.
+// All CTAs follow the same plan (computed from the step by each), so they meet
+// the same barriers.
 // ---------------------------------------------------------------------------
 constexpr int kRes3Ctas = 8;
 constexpr int kRes3Threads = 512;
@@ -804,8 +805,9 @@ int query_clusters3(const Args3& A, bool cmp64, int nct) {
 
 // CTAs of the resident cluster: 16 (a non-portable cluster size) where the
 // side splits into 16 slabs of at least two planes and the GPU can place
-// such a cluster, else 8.  At 32^3 the 16-CTA form takes 12.1 us per MC step
-// against 19.7 us with 8 CTAs (48^3: 31.5 / 57.9, 64^3: 66.7 / 127.4).
+// such a cluster, else 8.  At 32^3 the 16-CTA form took 12.1 us per MC step
+// against 19.7 us with 8 CTAs (48^3: 31.5 / 57.9, 64^3: 66.7 / 127.4; with 256
+// threads a CTA -- with 512 the 16-CTA form takes 8.9 at 32^3, 47.6 at 64^3).
 int resident3_ctas(const Args3& A, bool cmp64) {
   if (A.L % 16u == 0u && A.L >= 32u && query_clusters3(A, cmp64, 16) >= 1) return 16;
   return kRes3Ctas;
@@ -826,8 +828,8 @@ bool resident3_fits(const Args3& A, bool cmp64) {
 // The small-cube form of the automatic choice: up to 24^3 with any cluster, and
 // at 32^3 only when the 16-CTA cluster fits (with 8 CTAs it is slower there
 // than four launches per step).  The dataflow sweep runs these cubes too,
-// faster than the cluster (16^3 4.0 against 7.2 us per step, 24^3 4.1 against
-// 8.6, 32^3 4.0 against 8.8); the cluster remains for who asks for it.
+// faster than the cluster (16^3 4.0 against 7.3 us per step, 24^3 4.0 against
+// 8.7, 32^3 4.0 against 8.9); the cluster remains for who asks for it.
 bool resident3_auto(const Args3& A, bool cmp64) {
   if ((int)A.L > kRes3AutoSide || !resident3_fits(A, cmp64)) return false;
   return (int)A.L <= 24 || resident3_ctas(A, cmp64) == 16;

@@ -43,8 +43,10 @@ namespace {
 
 // Up to this many rows a thread the draws of a part are made before its first load
 // (they are the work there is while the neighbours' words come: 900^2 6.0 us per
-// step, 6.3 without; 1024^2 7.5 and 7.7); the draws of more rows do not fit the
-// registers.
+// step, 6.3 without; 1024^2 7.5 and 7.7); the draws of eight rows do not fit the
+// registers.  Nor do two words per update for four rows (152 bytes of spill stores
+// with 736 threads, 388 with 992): there 900^2 takes 8.3 us per step and 1024^2
+// 10.6, and 7.8 and 9.6 with the draws made after the loads.
 constexpr int kAheadRows = 4;
 // From this many rows on a warp rests between two looks at its neighbours' words:
 // the looks take instructions from the warps that sweep (ns; 1536^2 18.3 us per

@@ -843,25 +843,26 @@ int wave_scratch(cvf_handle* h, int shape) {
 // The automatic configuration of the lattices that the dataflow sweep does not
 // take (Flow2Plan; it is faster wherever it fits: 64^2 1.3 against 2.7 us per
 // step with the resident form, 258^2 2.0 / 7.9 tiled, 512^2 2.7 / 7.0 and 1024^2
-// 7.4 / 11.2 with the wavefront): the resident form for small lattices; the
+// 7.4 / 10.4 with the wavefront): the resident form for small lattices; the
 // wavefront sweep from 256^2 up, with the tiled sweep's shape rule (the
 // largest shape with at least as many tiles as the tiled sweep has resident
-// blocks: the fastest wavefront shape at 768^2, 1536^2, 2048^2 and from
-// 2560^2 up, within 1.2 % of it at 1024^2, where 32 x 32 words ran at 11.2
-// against 11.3 us per step); the tiled sweep with that shape where the
-// wavefront does not fit.
+// blocks: the fastest wavefront shape at 256^2 to 768^2, 1280^2 to 2048^2 and
+// from 2560^2 up; at 1024^2 its 16 x 32 words take 10.8 us per step against
+// 10.4 with 32 x 32, at 1152^2 12.2 / 11.2); the tiled sweep with that shape
+// where the wavefront does not fit.
 // Measured on GB300, us per MC step, wavefront against the best tiled shape:
-// 256^2 6.6 / 7.5, 320^2 6.4 / 7.5, 384^2 7.0 / 7.4, 448^2 7.3 / 8.1,
-// 512^2 7.6 / 8.3, 1024^2 11.3 / 14.3, 2048^2 31.8 / 36.8, 3072^2 61.8 /
-// 71.3, 4096^2 103.0 / 115.0, 6144^2 226.6 / 248.9, 8192^2 402.3 / 428.5,
-// 12288^2 902.9 / 941.6, 16384^2 1603.5 / 1656.9 (the tiled sweep's partly
-// filled last round of tiles costs less the more tiles a step has, but the
-// wavefront stays ahead).
+// 256^2 6.4 / 7.2, 384^2 6.4 / 7.2, 448^2 6.6 / 7.7, 768^2 7.3 / 10.3, 1024^2
+// 10.4 / 13.6, 1280^2 13.2 / 17.3, 1536^2 17.1 / 21.4, 2048^2 28.4 / 35.0,
+// 2560^2 39.2 / 47.6, 3072^2 52.4 / 61.6, 4096^2 87.5 / 99.6, 5120^2 135.1 /
+// 155.5, 6144^2 193.5 / 213.3, 8192^2 341.7 / 365.0, 12288^2 765 / 802, 16384^2
+// 1357 / 1408 (512^2 7.7 / 7.7; the tiled sweep's partly filled last round of
+// tiles costs less the more tiles a step has, but the wavefront stays ahead).
 constexpr int kWaveAutoMin = 256;
 // The layered schedule runs as a dataflow sweep (cvf_flow2.cu) up to this side:
-// it is faster than a launch per segment at every side measured (1024^2 14.0
-// against 31.8 us per step, 2048^2 54.1 / 80.2, 4096^2 195 / 260), but its copy
-// doubles the lattice's memory (4 bytes a cell).
+// it is faster than a launch per segment at every side measured (64^2 3.6 against
+// 11.4 us per step, 512^2 4.4 / 14.3, 1024^2 14.1 / 30.0, 2048^2 53.7 / 78.2,
+// 4096^2 203 / 278, 8192^2 830 / 1062), but its copy doubles the lattice's memory
+// (4 bytes a cell).
 constexpr int kFlowLayerMaxSide = 16384;
 int auto_config(const cvf_handle* h) {
   const cvf_params& p = h->p;

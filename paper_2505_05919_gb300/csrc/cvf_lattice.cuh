@@ -19,14 +19,15 @@ constexpr int kTileWords = 64;
 // single-lattice tiled sweep; four (64 registers) for the batched kernel,
 // which keeps its item's replica state across the colour phases (the 256
 // replicas of the batched workload: 140.8 against 148.3 us per step on the
-// 64 x 64-word tiles the autotuner picks)
+// 64 x 64-word tiles the autotuner picks, both with an arm rule of 169
+// instructions a cell; 112 with the present one)
 constexpr int kSweepBlocksPerSM = 5;
 constexpr int kBatchBlocksPerSM = 4;
 // the wavefront sweep keeps more state across its items (the item, its
 // dependencies, the counts not yet reported): four blocks per SM at 64
 // registers (at five blocks, 48 registers, its column-walking form spills
 // about 220 bytes and runs 6 % slower at 4096^2: 115.9 against 108.6 us per
-// step)
+// step with that earlier rule; 87.5 with the present one)
 constexpr int kWaveBlocksPerSM = 4;
 
 struct LatticeArgs {

@@ -101,7 +101,8 @@ __device__ __forceinline__ uint32_t twice(uint32_t word, bool hi) {
 // sigma' each (169 -> 143 thread instructions a cell, ALU 73 -> 61 operations,
 // shared-memory wavefronts 38 -> 36): 4096^2 89.4 against 104.1 us per step,
 // 256 mixed replicas 109.8 against 151.5 (97.4 and 140.6 before the second
-// copy of the rows and the folded complement).
+// copy of the rows and the folded complement; 4096^2 87.5 with four row pairs per
+// walking iteration).
 template <bool CMP64, int ARM>
 __device__ __forceinline__ uint32_t update_arm2(uint32_t w2, uint32_t p2, uint32_t u, uint32_t k,
                                                 uint32_t q, const Tables2& Tb, uint32_t& pk) {
@@ -166,9 +167,9 @@ __device__ __forceinline__ void draws(uint32_t c, uint32_t s_lo, uint32_t s_hi,
 // (step_draw): the draws take 18 widening multiplies per cell instead of 20
 // (the wavefront sweep and the batched kernel, which have the registers for
 // the keys: 4096^2 104.7 against 106.7 us per step, 2048^2 32.2 against
-// 33.8; the tiled sweep, whose partly filled last round of tiles takes up
-// the cycles saved, ran 2 % slower with the folded rounds and keeps
-// KeysRound).  The step words passed with it are not used again.
+// 33.8, before update_arm2's present form; the tiled sweep, whose partly filled
+// last round of tiles takes up the cycles saved, ran 2 % slower with the folded
+// rounds and keeps KeysRound).  The step words passed with it are not used again.
 struct KeysStep {
   RoundKeys K;
   StepDraw sd;

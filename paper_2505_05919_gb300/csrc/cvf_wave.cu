@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, kWaveBlocksPerSM)
       // 64 x 64-word tiles: one TMA box (issued by thread 0) when the tile
       // and its halo lie inside the lattice (the box's x, p0 - 4, is a
       // multiple of 4 words); at 4096^2 106.7 against 108.6 us per step with
-      // cp.async.  The smaller tiles keep the 16-byte cp.async copies, which
+      // cp.async (before update_arm2's present form).  The smaller tiles keep the 16-byte cp.async copies, which
       // ran 1-2 % faster there (1024^2 with 16 x 32 words: 11.2 against
       // 11.4 us; 2048^2 with 32 x 32: 32.8 against 33.3).
       next_tma = TR >= 64 && A.use_tma && gn.th == TR && gn.tw == TW && gn.p0 >= 4 &&
