@@ -464,20 +464,22 @@ def measure_cubic(args, rank, world):
     per_step = statistics.median(ms)
     dev_s = dist.max_over_ranks(per_step / 1e3)
     o = lat.observables()
+    launches = lat.form() == "launches"  # (a small --L3: one launch per call)
     lat.close()
     upd = 6.0 * L ** 3
     out = {"value": upd * world / (dev_s * 1e9), "unit": UNIT, "L": L, "N": L ** 3,
            "ms_per_mc_step": dev_s * 1e3, "sweeps_timed": S,
            "paper_ms_per_mc_step": PAPER_3D_MS_PER_STEP_260 if L == 260 else None,
            "paper_hardware": "RTX 3060 (sm_86), cuRAND and copies included",
-           "launches_per_mc_step": 5,
+           "launches_per_mc_step": 5 if launches else 1 / S,
            "roofline": {"bound": "alu", "achieved": upd / (per_step * 1e6),
                         "peak": args.philox_ceiling, "unit": "sigma-updates/ns",
                         "frac": upd / (per_step * 1e6) / args.philox_ceiling if args.philox_ceiling else None,
                         "peak_kind": "measured: the Philox draws alone (cvf_philox_probe, four "
                                      "updates per Philox block, as the passes draw them)",
                         "traffic": None,
-                        "kernel": "k_eta3 + k_pass3 (five launches per MC step)"},
+                        "kernel": "k_eta3 + k_pass3 (five launches per MC step)" if launches
+                                  else "k_flow3 (one launch per call)"},
            "eta_moves": 1,
            "acceptance": o["acc_sigma"] / max(1.0, upd * o["sweep"]),
            "workload": "CVF 3D cubic lattice L=%d q=6, layered six-arm schedule with the eta "
